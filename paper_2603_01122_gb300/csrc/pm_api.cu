@@ -60,6 +60,7 @@ struct pm_batch {
     size_t items_cap = 0;
     int *d_meta = nullptr; // [0] tiles, [1] humans
     unsigned *d_head = nullptr;
+    pm::FastRow *d_fast = nullptr; // rows of the closed-form draw, kFastMaxB * S per human (NULL: not used)
     float *d_post_part = nullptr;
     unsigned *d_post_ticket = nullptr;
     float2 *d_prev = nullptr;        // [max_humans] start of the last prediction per slot (NaN: none), then a ticket word
@@ -274,6 +275,28 @@ void fill_rollout_tables(const pm_model *m, pm::RolloutArgs &a)
     a.B = m->B;
     a.goals = m->goals;
     a.beta = m->beta;
+    const double half = 3.14159265358979323846 / m->K;
+    a.fc.cK = (float)std::cos(half);
+    a.fc.sK = (float)std::sin(half);
+    a.fc.K2pi = (float)(0.5 / half);
+    a.fc.K = (float)m->K;
+}
+
+// What builds the closed-form draw's rows at `rows`; rows == NULL (nothing to
+// build) where the control set does not take that draw.
+pm::FastPrep fast_prep(const pm_model *m, const pm::RolloutArgs &a, pm::FastRow *rows)
+{
+    pm::FastPrep f;
+    std::memset(&f, 0, sizeof f);
+    f.beta = m->beta;
+    f.B = m->B;
+    f.S = a.tab.S > 0 ? a.tab.S : 1;
+    f.K = m->K;
+    f.w1 = m->w1;
+    f.w2 = m->w2;
+    for (int q = 0; q < f.S; ++q) f.sl[q] = a.tab.S > 0 ? a.tab.sl[q] : a.tab.s;
+    f.rows = pm::fast_applies(m->K, a.enabled, a.tab.S) ? rows : nullptr;
+    return f;
 }
 
 // The speed set of the belief update and the adjoint (S = 0: one speed).
@@ -334,10 +357,14 @@ pm_status ensure_stage(pm_ctx *ctx, size_t bytes)
 // Word 3 of the context's counter block is its device status word.
 unsigned *status_word(pm_ctx *ctx) { return ctx->ticket ? ctx->ticket + 3 : nullptr; }
 
+// The context's rows of the closed-form draw (kFastMaxB * PM_MAX_SPEEDS).
+pm::FastRow *fast_rows(pm_ctx *ctx) { return reinterpret_cast<pm::FastRow *>(ctx->ticket + 64); }
+
 pm_status ensure_posterior_scratch(pm_ctx *ctx, size_t bytes)
 {
     if (!ctx->ticket) {
-        cudaError_t e = cudaMalloc((void **)&ctx->ticket, 256);
+        // the counter block, then the rows of the closed-form draw
+        cudaError_t e = cudaMalloc((void **)&ctx->ticket, 256 + sizeof(pm::FastRow) * pm::kFastMaxB * PM_MAX_SPEEDS);
         if (e == cudaSuccess) e = cudaMemset(ctx->ticket, 0, 256);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -422,9 +449,11 @@ pm_status predict_impl(pm_ctx *ctx, const pm_model *model, const float *log_beli
     const size_t words = hist ? (size_t)grid->W * (size_t)grid->H * (size_t)horizon : 0;
     // (the rollout leaves its chunk counter at zero; without `zero` the
     // caller has zeroed the outputs)
-    cudaError_t ez = zero ? pm::launch_zero_outputs(hist ? counts : nullptr, words, hist ? oob : nullptr, horizon,
-                                                    head, ctx->sm_count, stream)
-                          : cudaSuccess;
+    const pm::FastPrep fp = fast_prep(model, a, model->B <= pm::kFastMaxB ? fast_rows(ctx) : nullptr);
+    a.fast = fp.rows;
+    const bool z = zero && hist;
+    cudaError_t ez = pm::launch_zero_outputs(z ? counts : nullptr, words, z ? oob : nullptr, horizon,
+                                             zero ? head : nullptr, ctx->sm_count, fp, stream);
     if (ez != cudaSuccess) return cuda_fail(ez, "zeroing counts, oob and the chunk counter");
     cudaError_t e = pm::launch_rollout(a, head, ctx->sm_count, stream);
     if (e != cudaSuccess) return cuda_fail(e, "rollout launch");
@@ -788,6 +817,13 @@ pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream)
     a.win_radius_cap = batch_radius_cap(b->window_kib, b->threads);
     a.status = status_word(ctx);
     a.marks = (b->block_flags && b->warp_hist && b->d_flags) ? 1 : 0;
+    a.fc = t.fc;
+    if (b->d_fast && b->warp_hist) {
+        a.fast = b->d_fast;
+        e = pm::launch_batch_fast_rows(b->d_humans, b->d_meta + 1, b->max_humans, fast_prep(&b->shared, t, b->d_fast),
+                                       stream);
+        if (e != cudaSuccess) return cuda_fail(e, "rows of the closed-form draw");
+    }
     const size_t dyn = batch_dyn_smem(b);
     int occ = b->occ;
     if (occ < 1)
@@ -983,7 +1019,8 @@ pm_status pm_zero_occupancy(pm_ctx *ctx, int32_t horizon, const pm_grid *grid, u
     if (st != PM_OK) return st;
     DeviceScope dev(ctx->device);
     const size_t words = (size_t)grid->W * (size_t)grid->H * (size_t)horizon;
-    cudaError_t e = pm::launch_zero_outputs(counts, words, oob, horizon, nullptr, ctx->sm_count, (cudaStream_t)stream);
+    cudaError_t e = pm::launch_zero_outputs(counts, words, oob, horizon, nullptr, ctx->sm_count, pm::FastPrep{},
+                                            (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "zeroing counts and oob");
     return PM_OK;
 }
@@ -1199,6 +1236,9 @@ pm_status pm_batch_create(pm_ctx *ctx, const pm_model *shared, int32_t max_human
     if (e == cudaSuccess) e = cudaMalloc(&b->d_meta, 256);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_srcs, (size_t)max_humans * sizeof(pm::SmoothSrc));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_head, 256);
+    if (e == cudaSuccess && pm::fast_applies(shared->K, enabled_mask(shared), multi_speed(shared) ? shared->n_speeds : 1))
+        e = cudaMalloc(&b->d_fast, (size_t)max_humans * pm::kFastMaxB * (multi_speed(shared) ? shared->n_speeds : 1) *
+                                       sizeof(pm::FastRow));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_post_part, (size_t)max_humans * b->post_stride * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_post_ticket, (size_t)max_humans * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(b->d_post_ticket, 0, (size_t)max_humans * sizeof(unsigned));
@@ -1232,6 +1272,7 @@ void pm_batch_destroy(pm_batch *b)
     cudaFree(b->d_srcs);
     cudaFree(b->d_flags);
     cudaFree(b->d_head);
+    cudaFree(b->d_fast);
     cudaFree(b->d_post_part);
     cudaFree(b->d_post_ticket);
     cudaFree(b->d_prev);

@@ -131,13 +131,13 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 3) batch_rollout_kernel(cons
     }
 }
 
-// Bytes of one warp's tables in dynamic shared memory: comp[kMaxJ] (16 B
-// each) then cdf[kMaxJ] (4 B each). Sized for the library's largest G*B, not
+// Bytes of one warp's tables in dynamic shared memory: the random words, then
+// comp[kMaxJ] (16 B each), then cdf[kMaxJ] (4 B each). Sized for the library's largest G*B, not
 // for the current batch, so that a CUDA graph captured on one batch stays
 // valid when humans with more components join later.
-constexpr size_t kWarpTableBytes = (size_t)kMaxJ * 20;
+constexpr size_t kWarpTableBytes = (size_t)kMaxJ * 20 + kWarpWords * 4;
 // Several speeds: also the components' beta[kMaxJ] (4 B each) after cdf.
-constexpr size_t kWarpTableBytesMS = (size_t)kMaxJ * 24;
+constexpr size_t kWarpTableBytesMS = (size_t)kMaxJ * 24 + kWarpWords * 4;
 
 // Persistent warps over all humans: each warp takes a 32-particle tile
 // (human, first particle) from the global counter, loads that human's
@@ -148,7 +148,7 @@ constexpr size_t kWarpTableBytesMS = (size_t)kMaxJ * 24;
 // MS: the control set of several speeds (draw_multi).
 // MARKS: also write the block occupancy flags (a separate instantiation, so
 // the kernel without marks carries none of their code).
-template <int KT, bool FULL, bool MS = false, bool MARKS = false>
+template <int KT, bool FULL, bool MS = false, bool MARKS = false, bool FAST = false>
 __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
 {
     __shared__ float2 step[MS ? PM_MAX_SPEEDS * kMaxK : kMaxK];
@@ -162,6 +162,8 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
     }
     __syncthreads();
     char *slab = reinterpret_cast<char *>(dyn) + (size_t)warp * (MS ? kWarpTableBytesMS : kWarpTableBytes);
+    uint32_t *words = reinterpret_cast<uint32_t *>(slab) + lane;
+    slab += kWarpWords * 4;
     float4 *comp = reinterpret_cast<float4 *>(slab);
     uint32_t *cdf = reinterpret_cast<uint32_t *>(slab + (size_t)kMaxJ * 16);
     float *betas = reinterpret_cast<float *>(slab + (size_t)kMaxJ * 20); // MS only
@@ -223,12 +225,14 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
         c.tr_states = nullptr;
         c.tr_head = nullptr;
         c.tr_comp = nullptr;
+        c.B = h->B;
+        c.fast = (a.fast && h->B <= kFastMaxB) ? a.fast + (size_t)item.x * kFastMaxB * (MS ? a.tab.S : 1) : nullptr;
         c.flags = MARKS ? h->flags : nullptr;
         c.fbx = h->fbx;
         c.fplane = h->fbx * h->fby;
         if constexpr (MS)
-            rollout_lane<KT, false, true>(a.tab, a.enabled, a.s2, c, comp, cdf, step, betas, a.K, h->speed_on);
-        else rollout_lane<KT, FULL>(a.tab, a.enabled, a.s2, c, comp, cdf, step);
+            rollout_lane<KT, false, true, true, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words, betas, a.K, h->speed_on);
+        else rollout_lane<KT, FULL, false, FAST, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words);
     }
 }
 
@@ -236,10 +240,18 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
 // per SM), and 72 (7 CTAs) for the one-speed instantiations with K <= 36,
 // which do not spill there (24 bytes with marks); the 64-human served frame
 // is 0.6 % faster with 7. K = 64 and several speeds spill at 72 and keep 80.
-template <int KT, bool FULL, bool MS = false, bool MARKS = false>
+template <int KT, bool FULL, bool MARKS = false>
 __global__ void __launch_bounds__(kBatchMaxThreads, 3) batch_warp_kernel(const __grid_constant__ BatchArgs a)
 {
-    batch_warp_body<KT, FULL, MS, MARKS>(a);
+    batch_warp_body<KT, FULL, false, MARKS>(a);
+}
+
+// With the closed-form draw. One speed, K <= 36: 80 registers (6 CTAs of 128
+// threads per SM); K = 64 and several speeds: 96 (5 CTAs), fewer spills.
+template <int KT, bool FULL, bool MS, bool MARKS>
+__global__ void __maxnreg__((MS || KT == 64) ? 96 : 80) batch_fast_kernel(const __grid_constant__ BatchArgs a)
+{
+    batch_warp_body<KT, FULL, MS, MARKS, true>(a);
 }
 
 template <int KT, bool FULL, bool MARKS = false>
@@ -395,12 +407,47 @@ __global__ void batch_zero_reach_kernel(const BatchHuman *humans, const int *n_d
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
+// Rows of the closed-form draw: kRowsPerCta groups of kFastGroup threads, a
+// row each, from row0 on.
+constexpr int kRowThreads = 256, kRowsPerCta = kRowThreads / kFastGroup;
+
+__device__ __forceinline__ void build_rows(const FastPrep &fp, int row0)
+{
+    __shared__ FastWork ws[kRowsPerCta];
+    const int grp = threadIdx.x / kFastGroup, row = row0 + grp, n = fp.B * fp.S;
+    fast_row_build(fp, min(row, n - 1), row < n, ws[grp], threadIdx.x - grp * kFastGroup, kFastGroup);
+}
+
+// blockIdx.y strides over the humans, the x dimension covers kFastMaxB * S rows.
+__global__ void __launch_bounds__(kRowThreads) batch_fast_rows_kernel(const BatchHuman *humans, const int *n_dev,
+                                                                      const __grid_constant__ FastPrep fp)
+{
+    const int n = *n_dev;
+    for (int hh = blockIdx.y; hh < n; hh += gridDim.y) {
+        const BatchHuman &h = humans[hh];
+        FastPrep p = fp;
+        p.B = h.B;
+        p.beta = h.beta;
+        p.rows = fp.rows + (size_t)hh * kFastMaxB * fp.S;
+        const int row0 = blockIdx.x * kRowsPerCta;
+        if (h.B <= kFastMaxB && row0 < h.B * fp.S) build_rows(p, row0); // the same for the whole CTA
+    }
+}
+
 // The single-human form of the above: the counts in 16-byte words (scalar
 // head and tail), oob and the chunk counter, so one launch replaces three
 // memsets before the rollout.
-__global__ void zero_outputs_kernel(uint32_t *counts, size_t words, uint32_t *oob, int T, unsigned *head)
+// The CTAs from zblocks on build the rows of the closed-form draw instead,
+// kRowsPerCta each, while the others write.
+__global__ void __launch_bounds__(kRowThreads) zero_outputs_kernel(uint32_t *counts, size_t words, uint32_t *oob, int T,
+                                                                   unsigned *head, int zblocks,
+                                                                   const __grid_constant__ FastPrep fp)
 {
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    if ((int)blockIdx.x >= zblocks) {
+        build_rows(fp, ((int)blockIdx.x - zblocks) * kRowsPerCta);
+        return;
+    }
+    const size_t stride = (size_t)zblocks * blockDim.x;
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (counts) {
         const size_t lead0 = ((16 - ((uintptr_t)counts & 15)) & 15) / 4;
@@ -434,12 +481,21 @@ template <int KT, bool FULL>
 cudaError_t batch_shape(const BatchArgs &a, const RolloutShape &sh, int blocks, size_t dyn, cudaStream_t s, int *occ)
 {
     if (sh.warp_hist) {
-        if constexpr (KT <= 36) {
+        if constexpr (KT >= kFastMinK) {
+            if (FULL || fast_applies(a.K, a.enabled, 1)) {
+                if (a.marks)
+                    return launch_or_query(batch_fast_kernel<KT, FULL, false, true>, a, blocks, sh.threads, dyn, s, occ);
+                return launch_or_query(batch_fast_kernel<KT, FULL, false, false>, a, blocks, sh.threads, dyn, s, occ);
+            }
+        }
+        if constexpr (FULL && KT >= kFastMinK) {
+            return cudaErrorInvalidValue; // not reached: taken above
+        } else if constexpr (KT <= 36) {
             if (a.marks) return launch_or_query(batch_warp_kernel72<KT, FULL, true>, a, blocks, sh.threads, dyn, s, occ);
             return launch_or_query(batch_warp_kernel72<KT, FULL>, a, blocks, sh.threads, dyn, s, occ);
         } else {
             if (a.marks)
-                return launch_or_query(batch_warp_kernel<KT, FULL, false, true>, a, blocks, sh.threads, dyn, s, occ);
+                return launch_or_query(batch_warp_kernel<KT, FULL, true>, a, blocks, sh.threads, dyn, s, occ);
             return launch_or_query(batch_warp_kernel<KT, FULL>, a, blocks, sh.threads, dyn, s, occ);
         }
     }
@@ -451,17 +507,17 @@ cudaError_t batch_dispatch(const BatchArgs &a, const RolloutShape &sh, int block
     if (a.tab.S > 0) { // several speeds: warp-combined emplacement only
         switch (a.K) {
         case 16:
-            return a.marks ? launch_or_query(batch_warp_kernel<16, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_warp_kernel<16, false, true>, a, blocks, sh.threads, dyn, s, occ);
+            return a.marks ? launch_or_query(batch_fast_kernel<16, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
+                           : launch_or_query(batch_fast_kernel<16, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
         case 32:
-            return a.marks ? launch_or_query(batch_warp_kernel<32, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_warp_kernel<32, false, true>, a, blocks, sh.threads, dyn, s, occ);
+            return a.marks ? launch_or_query(batch_fast_kernel<32, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
+                           : launch_or_query(batch_fast_kernel<32, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
         case 36:
-            return a.marks ? launch_or_query(batch_warp_kernel<36, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_warp_kernel<36, false, true>, a, blocks, sh.threads, dyn, s, occ);
+            return a.marks ? launch_or_query(batch_fast_kernel<36, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
+                           : launch_or_query(batch_fast_kernel<36, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
         default:
-            return a.marks ? launch_or_query(batch_warp_kernel<0, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_warp_kernel<0, false, true>, a, blocks, sh.threads, dyn, s, occ);
+            return a.marks ? launch_or_query(batch_fast_kernel<0, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
+                           : launch_or_query(batch_fast_kernel<0, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
         }
     }
     const int KT = rollout_kt_for(a.K);
@@ -503,7 +559,7 @@ cudaError_t launch_batch_rollout(const BatchArgs &a, const RolloutShape &shape, 
 }
 
 cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, int T, unsigned *head, int sm_count,
-                                cudaStream_t s)
+                                const FastPrep &fp, cudaStream_t s)
 {
     // enough threads for a few 16-byte stores each at paper-scale sizes,
     // never more than the work
@@ -512,7 +568,19 @@ cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, i
     const size_t cap = (size_t)(sm_count > 0 ? sm_count : 1) * 4;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    zero_outputs_kernel<<<(unsigned)blocks, 256, 0, s>>>(counts, words, oob, T, head);
+    if (!counts && !oob && !head) blocks = 0;
+    const unsigned rows = fp.rows ? (fp.B * fp.S + kRowsPerCta - 1) / kRowsPerCta : 0;
+    if (blocks + rows == 0) return cudaSuccess;
+    zero_outputs_kernel<<<(unsigned)blocks + rows, kRowThreads, 0, s>>>(counts, words, oob, T, head, (int)blocks, fp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batch_fast_rows(const BatchHuman *humans, const int *n_dev, int max_rows, const FastPrep &fp,
+                                   cudaStream_t s)
+{
+    if (max_rows <= 0) return cudaSuccess;
+    const dim3 grid((kFastMaxB * fp.S + kRowsPerCta - 1) / kRowsPerCta, (unsigned)std::min(max_rows, 1024));
+    batch_fast_rows_kernel<<<grid, kRowThreads, 0, s>>>(humans, n_dev, fp);
     return cudaGetLastError();
 }
 

@@ -181,6 +181,14 @@ __device__ __forceinline__ void flag_status(unsigned *status, unsigned bit)
     if (status) atomicOr(status, bit);
 }
 
+// Constants of the closed-form draw over K equally spaced headings.
+struct FastRow;
+struct FastConst {
+    float cK, sK; // cos, sin of pi / K
+    float K2pi;   // K / (2 pi)
+    float K;
+};
+
 // Arguments of the rollout kernel (Algorithm 1 + emplacement).
 struct RolloutArgs {
     HeadingTab tab;
@@ -202,6 +210,8 @@ struct RolloutArgs {
     uint32_t *oob;
     int win_x0, win_y0;  // shared-memory window origin (grid cells)
     int win_side;        // window width | height << 16 (cells, each <= 255); 0 = no window
+    FastConst fc;
+    const FastRow *fast; // rows of the closed-form draw (b * S + q), or NULL
     int n_trace;
     float *tr_states;
     uint8_t *tr_head;

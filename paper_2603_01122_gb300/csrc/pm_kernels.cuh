@@ -4,6 +4,7 @@
 // pieces are in pm_internal.cuh.
 #pragma once
 
+#include "pm_fastdraw.cuh"
 #include "pm_internal.cuh"
 
 namespace pm {
@@ -174,6 +175,8 @@ struct BatchArgs {
     int win_radius_cap;  // (2r+1)^2 cells fit the dynamic shared memory
     unsigned *status;    // context status word (or NULL)
     int marks;           // write block occupancy flags (the humans' flags are set)
+    FastConst fc;
+    const FastRow *fast; // kFastMaxB * S rows per human (S = 1: one speed), or NULL
 };
 
 // Launch shape of the rollout: threads per CTA, particles per thread (1 or
@@ -211,10 +214,15 @@ cudaError_t launch_batch_rollout(const BatchArgs &a, const RolloutShape &shape, 
 // size the grid only.
 cudaError_t launch_batch_zero(const BatchHuman *humans, const int *n_dev, int max_rows, int sm_count, int t_max,
                               float2 *prev, unsigned *ticket, float smax, cudaStream_t s);
-// One human's outputs before its rollout, in one launch: counts [words]
-// (or NULL), oob [T] (or NULL) and the chunk counter.
+// What one human's rollout needs first, in one launch: counts [words] (or
+// NULL) and oob [T] (or NULL) zeroed, the chunk counter reset, and the rows of
+// the closed-form draw (fp.rows, or NULL).
 cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, int T, unsigned *head, int sm_count,
-                                cudaStream_t s);
+                                const FastPrep &fp, cudaStream_t s);
+// The rows of every human of a batch with at most kFastMaxB beta values
+// (fp: B and beta per human).
+cudaError_t launch_batch_fast_rows(const BatchHuman *humans, const int *n_dev, int max_rows, const FastPrep &fp,
+                                   cudaStream_t s);
 size_t adjoint_scratch_bytes(int M, int G, int J);
 void adjoint_scratch_layout(void *base, int M, int G, int J, AdjointArgs &a);
 

@@ -19,7 +19,7 @@
 // is binned with FP32 operations (x - x0) * inv_res and the lanes of the warp
 // that land in the same cell are combined (match.any) into one global
 // reduction per cell and step.
-// rollout_multi_kernel<KT> is the same kernel for a control set of several
+// rollout_multi_kernel<KT, TRACE> is the same kernel for a control set of several
 // speeds (controls = speeds x headings, Sec. IV-B): the fused per-speed draw
 // for K = KT, the general one for any K (KT = 0).
 #include <cuda_runtime.h>
@@ -53,13 +53,14 @@ __device__ __forceinline__ void release_counter(unsigned *head, int lane)
 // takes chunks of 32 particles (one per lane) from a global counter until the
 // particles are exhausted, so the work spreads evenly over the schedulers and
 // SMs whatever the particle count.
-template <int KT, bool FULL>
-__global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
+template <int KT, bool FULL, bool FAST, bool TRACE>
+__global__ void __launch_bounds__(kWarpCtaThreads, (FAST && KT == 64) ? 5 : kWarpCtaMinBlocks)
     rollout_warp_kernel(const __grid_constant__ RolloutArgs a, unsigned *head)
 {
     __shared__ float4 comp[kMaxJ];
     __shared__ uint32_t cdf[kMaxJ];
     __shared__ float2 step[kMaxK];
+    __shared__ uint32_t words[kWarpCtaThreads / 32 * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31;
     const int J = a.G * a.B;
     for (int j = tid; j < J; j += blockDim.x) {
@@ -95,6 +96,8 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     c.tr_states = a.tr_states;
     c.tr_head = a.tr_head;
     c.tr_comp = a.tr_comp;
+    c.fast = a.fast;
+    c.B = a.B;
     c.flags = nullptr;
     c.fbx = c.fplane = 0;
     for (;;) {
@@ -104,14 +107,14 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
         const int64_t i0 = (int64_t)item * 32;
         if (i0 >= a.N) break;
         c.i = i0 + lane;
-        rollout_lane<KT, FULL>(a.tab, a.enabled, a.s2, c, comp, cdf, step);
+        rollout_lane<KT, FULL, false, FAST, TRACE>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words + (tid >> 5) * kWarpWords + lane);
     }
     release_counter(head, lane);
 }
 
 // The same persistent warps for a control set of several speeds: KT > 0 is
 // the heading count of the fused draw (K == KT), KT = 0 the general draw.
-template <int KT>
+template <int KT, bool TRACE>
 __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     rollout_multi_kernel(const __grid_constant__ RolloutArgs a, unsigned *head)
 {
@@ -119,6 +122,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     __shared__ float betas[kMaxJ];
     __shared__ uint32_t cdf[kMaxJ];
     __shared__ float2 step[PM_MAX_SPEEDS * kMaxK];
+    __shared__ uint32_t words[kWarpCtaThreads / 32 * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31;
     const int J = a.G * a.B;
     for (int j = tid; j < J; j += blockDim.x) {
@@ -156,6 +160,8 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     c.tr_states = a.tr_states;
     c.tr_head = a.tr_head;
     c.tr_comp = a.tr_comp;
+    c.fast = a.fast;
+    c.B = a.B;
     c.flags = nullptr;
     c.fbx = c.fplane = 0;
     for (;;) {
@@ -165,16 +171,16 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
         const int64_t i0 = (int64_t)item * 32;
         if (i0 >= a.N) break;
         c.i = i0 + lane;
-        rollout_lane<KT, false, true>(a.tab, a.enabled, a.s2, c, comp, cdf, step, betas, a.K, a.tab.speed_on);
+        rollout_lane<KT, false, true, true, TRACE>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words + (tid >> 5) * kWarpWords + lane, betas, a.K, a.tab.speed_on);
     }
     release_counter(head, lane);
 }
 
-template <int KT>
+template <int KT, bool TRACE>
 cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
     int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rollout_multi_kernel<KT>, kWarpCtaThreads, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rollout_multi_kernel<KT, TRACE>, kWarpCtaThreads, 0);
     if (e != cudaSuccess) return e;
     if (occ) {
         *occ = n;
@@ -185,16 +191,22 @@ cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cud
     int64_t blocks = (int64_t)sm_count * (n > 0 ? n : 1);
     if (need < blocks) blocks = need;
     cudaGetLastError();
-    rollout_multi_kernel<KT><<<(unsigned)blocks, kWarpCtaThreads, 0, s>>>(a, head);
+    rollout_multi_kernel<KT, TRACE><<<(unsigned)blocks, kWarpCtaThreads, 0, s>>>(a, head);
     return cudaGetLastError();
 }
 
-template <int KT>
+template <int KT, bool TRACE>
 cudaError_t launch_kt(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
+    // every heading enabled and K == KT: the FULL form, in closed form where
+    // K >= kFastMinK
+    const bool fast = fast_applies(a.K, a.enabled, 1);
+    auto k = rollout_warp_kernel<KT, false, false, TRACE>;
+    if constexpr (KT >= kFastMinK) {
+        if (fast) k = rollout_warp_kernel<KT, false, true, TRACE>;
+    }
     const uint64_t all = (KT >= 64) ? ~0ull : ((1ull << KT) - 1ull);
-    const bool full = (a.K == KT) && ((a.enabled & all) == all);
-    auto k = full ? rollout_warp_kernel<KT, true> : rollout_warp_kernel<KT, false>;
+    if (a.K == KT && (a.enabled & all) == all) k = rollout_warp_kernel<KT, true, (KT >= kFastMinK), TRACE>;
     int n = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kWarpCtaThreads, 0);
     if (e != cudaSuccess) return e;
@@ -211,21 +223,22 @@ cudaError_t launch_kt(const RolloutArgs &a, unsigned *head, int sm_count, cudaSt
     return cudaGetLastError();
 }
 
+template <bool TRACE>
 cudaError_t dispatch(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
     if (a.tab.S > 0) { // several speeds (all K headings enabled, K % 4 == 0)
         switch (a.K) {
-        case 16: return launch_multi<16>(a, head, sm_count, s, occ);
-        case 32: return launch_multi<32>(a, head, sm_count, s, occ);
-        case 36: return launch_multi<36>(a, head, sm_count, s, occ);
-        default: return launch_multi<0>(a, head, sm_count, s, occ);
+        case 16: return launch_multi<16, TRACE>(a, head, sm_count, s, occ);
+        case 32: return launch_multi<32, TRACE>(a, head, sm_count, s, occ);
+        case 36: return launch_multi<36, TRACE>(a, head, sm_count, s, occ);
+        default: return launch_multi<0, TRACE>(a, head, sm_count, s, occ);
         }
     }
     switch (rollout_kt_for(a.K)) {
-    case 8: return launch_kt<8>(a, head, sm_count, s, occ);
-    case 16: return launch_kt<16>(a, head, sm_count, s, occ);
-    case 36: return launch_kt<36>(a, head, sm_count, s, occ);
-    default: return launch_kt<64>(a, head, sm_count, s, occ);
+    case 8: return launch_kt<8, TRACE>(a, head, sm_count, s, occ);
+    case 16: return launch_kt<16, TRACE>(a, head, sm_count, s, occ);
+    case 36: return launch_kt<36, TRACE>(a, head, sm_count, s, occ);
+    default: return launch_kt<64, TRACE>(a, head, sm_count, s, occ);
     }
 }
 
@@ -243,7 +256,9 @@ size_t rollout_static_smem_estimate() { return sizeof(RolloutShared); }
 
 cudaError_t launch_rollout(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s)
 {
-    return dispatch(a, head, sm_count, s, nullptr);
+    // (a plain histogram call carries no trace code)
+    return a.n_trace > 0 || !a.counts ? dispatch<true>(a, head, sm_count, s, nullptr)
+                                      : dispatch<false>(a, head, sm_count, s, nullptr);
 }
 
 } // namespace pm

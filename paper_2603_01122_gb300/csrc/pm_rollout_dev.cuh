@@ -2,6 +2,7 @@
 // single-human and the batched rollout kernels (private to the library).
 #pragma once
 
+#include "pm_fastdraw.cuh"
 #include "pm_internal.cuh"
 
 namespace pm {
@@ -926,6 +927,8 @@ struct TileCtx {
     float *tr_states;
     uint8_t *tr_head;
     int32_t *tr_comp;
+    const FastRow *fast; // the human's rows of the closed-form draw (b * S + q), or NULL (rollout_lane)
+    int B;
     uint8_t *flags; // block occupancy [T][fby][fbx] (warp emplacement), or NULL
     int fbx;
     int fplane;     // fbx * fby
@@ -1097,19 +1100,28 @@ __device__ __forceinline__ void rollout_tile(const HeadingTab &tab, uint64_t ena
         li = (li == 2) ? 0 : li + 1;
     }
 }
+constexpr int kWarpWords = 8 * 32;
+
 // Algorithm 1 for the particle of one lane: the (beta, g) draw from the
 // belief table (comp, cdf), then T heading draws and Euler steps, each step
 // emplaced with the lanes of the warp that land in the same cell combined
 // (match.any) into one global reduction. Every lane of the warp must call
 // it with the same c.T (idle lanes pass c.i >= c.N). No block barrier.
-// MS: the control set of several speeds (betas holds each component's beta,
+// words: this lane's column of the warp's kWarpWords words of shared memory
+// (lane + 32 w, w < 8). MS: the control set of several speeds (betas holds each component's beta,
 // step the S*K Euler steps, K the headings, speed_on the enabled speeds); KT >
 // 0 is then K itself, with draw_multi_lb for the components it applies to,
 // and KT = 0 runs draw_multi for any K.
-template <int KT, bool FULL, bool MS = false>
-__device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t enabled, float s2, const TileCtx &c,
-                                             const float4 *comp, const uint32_t *cdf, const float2 *step,
-                                             const float *betas = nullptr, int K = 0, uint32_t speed_on = 0u)
+// FAST: every heading is enabled and K >= kFastMinK: the draw is taken in
+// closed form (pm_fastdraw.cuh) at the steps where the whole warp can (each
+// lane's row usable and its goal farther than the row's range), and weight by
+// weight for the lanes it leaves open and at every other step. A warp-wide
+// choice: with both forms in one step the warp would pay for both.
+template <int KT, bool FULL, bool MS, bool FAST, bool TRACE>
+__device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t enabled, float s2, const FastConst &fc,
+                                             const TileCtx &c, const float4 *comp, const uint32_t *cdf,
+                                             const float2 *step, uint32_t *words, const float *betas = nullptr, int K = 0,
+                                             uint32_t speed_on = 0u)
 {
     const int lane = threadIdx.x & 31;
     const uint64_t i = (uint64_t)c.i;
@@ -1119,6 +1131,11 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
     bool lb = false;
     // several speeds with exactly one enabled: its index (else -1)
     const int one_speed = (MS && __popc(speed_on) == 1) ? __ffs((int)speed_on) - 1 : -1;
+    // closed-form draw: the lane's row, the squared goal distance it needs and
+    // the part of the tolerance that grows with that distance
+    const FastRow *row = nullptr;
+    float fkap = 0.0f, ftol = 0.0f, ftol_r = 0.0f, fr2 = INFINITY;
+    bool wfast = false;
     if (act) {
         const U64x4 r = philox4x64_10(U64x4{i, 0ull, kPurposeSelect, 0ull}, c.seed, c.human);
         const uint32_t thr = (uint32_t)(((uint64_t)((uint32_t)r.a >> 8) * (uint64_t)cdf[c.J - 1]) >> 24);
@@ -1138,94 +1155,246 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
             cw = bt * tab.w1l[0]; // beta w1 v dt log2(e)
         }
         if (trc && c.tr_comp) c.tr_comp[i] = lo;
+        if constexpr (FAST) {
+            if (c.fast) {
+                row = c.fast + (size_t)(lo % c.B) * (MS ? tab.S : 1);
+                float rmin = 0.0f; // the goal distance below which a row no longer holds
+                if constexpr (MS) {
+                    for (int q = 0; q < tab.S; ++q)
+                        if ((speed_on >> q) & 1u) {
+                            const float rm = row[q].rho_max;
+                            rmin = fmaxf(rmin, rm > 0.0f ? row[q].s / rm : INFINITY);
+                            ftol_r = fmaxf(ftol_r, fabsf(row[q].kappa) / row[q].s);
+                        }
+                } else {
+                    rmin = row->rho_max > 0.0f ? row->s / row->rho_max : INFINITY;
+                    ftol_r = fabsf(row->kappa) / row->s;
+                    fkap = row->kappa;
+                    ftol = row->tol;
+                }
+                fr2 = rmin * rmin * 1.00001f;
+                // the weight-by-weight draw's exponents carry the rounding of
+                // beta w2 r: some 2^-24 of it after its residual correction
+                ftol_r *= 4e-10f;
+            }
+        }
+    }
+    if constexpr (FAST) {
+        wfast = __all_sync(0xffffffffu, !act || fr2 < INFINITY);
+        if (!act) row = c.fast; // an idle lane computes along (any row will do)
     }
     const size_t plane = (size_t)c.W * (size_t)c.H;
+    uint32_t *crow = c.counts; // step t's plane of the histogram
+    const int xbase = 0x4B400000 + c.cx_off, ybase = 0x4B400000 + c.cy_off;
+    // the 32 random bits of step t: a Philox block serves eight steps; beside
+    // the closed-form draw its words wait in this lane's column of `words`
+    // (held in registers they cost that loop spills), else in registers,
+    // shifted at each step
     uint32_t q0 = 0, q1 = 0, q2 = 0, q3 = 0, q4 = 0, q5 = 0, q6 = 0, q7 = 0;
-    for (int t = 1; t <= c.T; ++t) {
-        uint32_t key = 0xFFFFFFFFu; // idle lane
-        int fkey = 0;               // block of the cell (flags only)
-        int k = 0;
-        bool settle = false; // several speeds: the FP32 draw was too close to a CDF boundary
-        uint32_t word = 0u;
-        if (act) {
-            if (((t - 1) & 7) == 0) {
-                const U64x4 r = philox4x64_10(U64x4{i, (uint64_t)((t - 1) >> 3), kPurposeStep, 0ull}, c.seed, c.human);
+    auto next_word = [&](int t) {
+        if (((t - 1) & 7) == 0) {
+            const U64x4 r = philox4x64_10(U64x4{i, (uint64_t)((t - 1) >> 3), kPurposeStep, 0ull}, c.seed, c.human);
+            if constexpr (!FAST) {
                 q0 = (uint32_t)r.a; q1 = (uint32_t)(r.a >> 32);
                 q2 = (uint32_t)r.b; q3 = (uint32_t)(r.b >> 32);
                 q4 = (uint32_t)r.c; q5 = (uint32_t)(r.c >> 32);
                 q6 = (uint32_t)r.d; q7 = (uint32_t)(r.d >> 32);
-            }
-            word = q0;
-            q0 = q1; q1 = q2; q2 = q3; q3 = q4; q4 = q5; q5 = q6; q6 = q7;
-            if constexpr (MS) {
-                if constexpr (KT > 0) { // K == KT, all headings enabled: the fused form where it applies
-                    if (lb && one_speed >= 0) {
-                        // one enabled speed m (a human standing still keeps only the
-                        // slow one): ||z + s m e_k - g|| = m ||(z - g) / m + s e_k||, so
-                        // the one-speed draw at the scaled offset with cb m draws the
-                        // same policy (the speed term is common to every control)
-                        const float im = tab.inv_mult[one_speed], cbm = cb * tab.mult[one_speed];
-                        k = one_speed * KT +
-                            draw_heading_lb<KT>(tab, lb_step_d(tab, s2, (x - gx) * im, (y - gy) * im, cbm), cbm, word);
-                    } else if (lb) {
-                        k = draw_multi_lb<KT>(tab, speed_on, x, y, gx, gy, bt, cb, cw, word, settle);
-                    } else {
-                        k = draw_multi(tab, speed_on, K, x, y, gx, gy, bt, cb, cw, lb, word, settle);
-                    }
-                } else {
-                    k = draw_multi(tab, speed_on, K, x, y, gx, gy, bt, cb, cw, lb, word, settle);
-                }
             } else {
-                k = draw<KT, FULL>(tab, enabled, s2, x, y, gx, gy, cb, lb, word);
+                words[0 * 32] = (uint32_t)r.a; words[1 * 32] = (uint32_t)(r.a >> 32);
+                words[2 * 32] = (uint32_t)r.b; words[3 * 32] = (uint32_t)(r.b >> 32);
+                words[4 * 32] = (uint32_t)r.c; words[5 * 32] = (uint32_t)(r.c >> 32);
+                words[6 * 32] = (uint32_t)r.d; words[7 * 32] = (uint32_t)(r.d >> 32);
             }
         }
-        if constexpr (MS) {
-            // a draw too close to a CDF boundary for FP32 is settled in
-            // double-float by the whole warp, one flagged lane at a time
-            unsigned need = __ballot_sync(0xffffffffu, settle);
-            while (need) {
-                const int src = __ffs((int)need) - 1;
-                const int u = settle_multi_warp(tab, speed_on, K, x, y, gx, gy, bt, word, k, src);
-                if (lane == src) k = u;
-                need &= need - 1u;
-            }
+        if constexpr (!FAST) {
+            const uint32_t w = q0;
+            q0 = q1; q1 = q2; q2 = q3; q3 = q4; q4 = q5; q5 = q6; q6 = q7;
+            return w;
         }
-        if (act) {
-            const float2 st = step[k];
-            x = __fadd_rn(x, st.x);
-            y = __fadd_rn(y, st.y);
-            if (trc) {
+        return words[((t - 1) & 7) * 32];
+    };
+    // The Euler step along control k, the trace, and the cells of step t
+    // matched over the warp. The histogram add itself follows in flush(), at
+    // the next step's first wait: match.any takes long to answer, and nothing
+    // of the next draw depends on it. Idle lanes run along with their own key.
+    uint32_t pkey = 0u, ppeers = 0u;
+    int pfkey = 0;
+    auto flush = [&](int t) { // the adds of step t
+        if (TRACE && !c.hist) return;
+        // the lowest lane of each group of equal keys adds the group's size
+        if (pkey != 0xFFFFFFFFu && (ppeers & ((1u << lane) - 1u)) == 0u) {
+            const bool in = pkey != 0xFFFFFFFEu;
+            uint32_t *dst = in ? crow + pkey : c.oob + (t - 1);
+            red_add(dst, (uint32_t)__popc(ppeers));
+            if (c.flags && in) c.flags[(size_t)(t - 1) * c.fplane + pfkey] = 1u; // idempotent
+        }
+        crow += plane;
+    };
+    auto advance = [&](int t, int k) {
+        const float2 st = step[k];
+        x = __fadd_rn(x, st.x);
+        y = __fadd_rn(y, st.y);
+        if constexpr (TRACE) {
+            if (act && trc) {
                 const size_t o = (size_t)i * c.T + (t - 1);
                 if (c.tr_states) reinterpret_cast<float2 *>(c.tr_states)[o] = make_float2(x, y);
                 if (c.tr_head) c.tr_head[o] = (uint8_t)k;
             }
-            if (c.hist) {
-                const float vx = __fmul_rn(__fsub_rn(x, c.gx0), c.inv_res);
-                const float vy = __fmul_rn(__fsub_rn(y, c.gy0), c.inv_res);
-                // floor(v) for |v| < 2^22 on the FP32 pipe: v + 1.5 * 2^23 rounded
-                // down is exact and holds floor(v) in its low mantissa bits;
-                // larger |v| and NaN are outside every grid (W, H <= 2^22)
-                const int cx = (__float_as_int(__fadd_rd(vx, 12582912.0f)) - 0x4B400000) - c.cx_off;
-                const int cy = (__float_as_int(__fadd_rd(vy, 12582912.0f)) - 0x4B400000) - c.cy_off;
-                const bool in = fabsf(vx) < 4194304.0f && fabsf(vy) < 4194304.0f && cx >= 0 && cx < c.W &&
-                                cy >= 0 && cy < c.H;
-                key = in ? (uint32_t)(cy * c.W + cx) : 0xFFFFFFFEu;
-                if (c.flags) fkey = (cy >> kFlagShift) * c.fbx + (cx >> kFlagShift);
+            if (!c.hist) return;
+        }
+        const float vx = __fmul_rn(__fsub_rn(x, c.gx0), c.inv_res);
+        const float vy = __fmul_rn(__fsub_rn(y, c.gy0), c.inv_res);
+        // floor(v) for |v| < 2^22 on the FP32 pipe: v + 1.5 * 2^23 rounded
+        // down is exact and holds floor(v) in its low mantissa bits;
+        // larger |v| and NaN are outside every grid (W, H <= 2^22)
+        const int cx = __float_as_int(__fadd_rd(vx, 12582912.0f)) - xbase;
+        const int cy = __float_as_int(__fadd_rd(vy, 12582912.0f)) - ybase;
+        const bool in = fabsf(vx) < 4194304.0f && fabsf(vy) < 4194304.0f && (unsigned)cx < (unsigned)c.W &&
+                        (unsigned)cy < (unsigned)c.H;
+        pkey = in ? (uint32_t)(cy * c.W + cx) : 0xFFFFFFFEu;
+        pkey = act ? pkey : 0xFFFFFFFFu;
+        if (c.flags) pfkey = (cy >> kFlagShift) * c.fbx + (cx >> kFlagShift);
+        ppeers = __match_any_sync(0xffffffffu, pkey);
+    };
+    int t = 1, done = 0; // done: steps whose adds are made
+    while (t <= c.T) {
+        uint32_t word = 0u;
+        bool open = act;  // step t's draw is still to be made
+        bool have = false; // and its word is drawn
+        bool near = true; // several weight-by-weight steps follow
+        int k = 0;
+        if constexpr (FAST) {
+            if (wfast) {
+                // The closed-form steps, until one that the warp cannot take
+                // (a goal too close) or that some lanes leave open. The row's
+                // values live only in this loop: the weight-by-weight draw
+                // below needs the registers.
+                F2 fq[kFastD][kFastP];
+                if constexpr (!MS) fast_load(*row, fq);
+                for (; t <= c.T; ++t) {
+                    word = next_word(t);
+                    have = true;
+                    const float dx = x - gx, dy = y - gy, r2 = fmaf(dx, dx, dy * dy);
+                    const float ri = rsqrt_approx(r2);
+                    // 23 of the 24 bits, at the middle of the pair they leave open
+                    const float u = (__uint_as_float(0x3F800000u | (word >> 9)) - 1.0f) + 0x1p-25f;
+                    const float far = ftol_r * (r2 * ri);
+                    F2 P[kFastP];
+                    FastDraw w;
+                    const FastRow *o = row;
+                    float rho, kap = fkap, tol = ftol + far;
+                    int base = 0;
+                    if constexpr (MS) {
+                        float wq[PM_MAX_SPEEDS], total = 0.0f;
+#pragma unroll
+                        for (int q = 0; q < PM_MAX_SPEEDS; ++q) {
+                            wq[q] = 0.0f;
+                            if (q >= tab.S || !((speed_on >> q) & 1u)) continue; // the same for the whole warp
+                            const float rq = tab.sl[q] * ri;
+                            const float4 m = *reinterpret_cast<const float4 *>(row[q].a0);
+                            wq[q] = fmaf(fmaf(fmaf(m.w, rq, m.z), rq, m.y), rq, m.x);
+                            total += wq[q];
+                        }
+                        // the speed whose share of the total holds u, and the fraction of it below u
+                        const float v = u * total;
+                        float start = 0.0f, run = wq[0], wsel = wq[0];
+                        int sp = 0;
+#pragma unroll
+                        for (int q = 1; q < PM_MAX_SPEEDS; ++q) {
+                            const bool in = v >= run && wq[q] > 0.0f;
+                            sp = in ? q : sp;
+                            start = in ? run : start;
+                            wsel = in ? wq[q] : wsel;
+                            run += wq[q];
+                        }
+                        const float iw = fast_rcp(wsel);
+                        o = row + sp;
+                        base = sp * K;
+                        rho = o->s * ri;
+                        kap = o->kappa;
+                        tol = (2.0f * o->tol + far) * (total * iw); // (the mean weights carry the same error)
+                        fast_load(*o, fq);
+                        fast_poly(fq, rho, P);
+                        w = fast_begin(fc, P, dx * ri, dy * ri, (v - start) * iw, o->guess);
+                    } else {
+                        rho = tab.s * ri;
+                        fast_poly(fq, rho, P);
+                        w = fast_begin(fc, P, dx * ri, dy * ri, u, o->guess);
+                    }
+                    if (done < t - 1) {
+                        flush(t - 1);
+                        done = t - 1;
+                    }
+                    k = fast_step(fc, P, rho, kap, tol, w);
+                    open = act && (k < 0 || !(r2 > fr2));
+                    if (__any_sync(0xffffffffu, open)) {
+                        near = __any_sync(0xffffffffu, act && !(r2 > fr2));
+                        // where the table was coarse, once more from the better point
+                        if (!near && open && fabsf(w.dl) > 1e-4f) {
+                            k = fast_step(fc, P, rho, kap, tol, w);
+                            open = k < 0;
+                        }
+                        k += base;
+                        if (near || __any_sync(0xffffffffu, open)) break;
+                    } else {
+                        k += base;
+                    }
+                    advance(t, act ? k : 0);
+                }
+                if (t > c.T) break;
+                if (near) open = act; // every lane: the two forms in one step would cost both
             }
         }
-        if (c.hist) {
-            const uint32_t peers = __match_any_sync(0xffffffffu, key);
-            // the lowest lane of each group of equal keys adds the group's size
-            if (key != 0xFFFFFFFFu && (peers & ((1u << lane) - 1u)) == 0u) {
-                if (key == 0xFFFFFFFEu) {
-                    red_add(c.oob + (t - 1), (uint32_t)__popc(peers));
+        // weight by weight: this step's open lanes, and with a goal near (or
+        // without the closed form) the steps up to the next Philox block
+        do {
+            bool settle = false; // several speeds: the FP32 draw was too close to a CDF boundary
+            if (!have) {
+                word = next_word(t);
+                open = act;
+            }
+            have = false;
+            if (open) {
+                if constexpr (MS) {
+                    if constexpr (KT > 0) { // K == KT, all headings enabled: the fused form where it applies
+                        if (lb && one_speed >= 0) {
+                            // one enabled speed m (a human standing still keeps only the
+                            // slow one): ||z + s m e_k - g|| = m ||(z - g) / m + s e_k||, so
+                            // the one-speed draw at the scaled offset with cb m draws the
+                            // same policy (the speed term is common to every control)
+                            const float im = tab.inv_mult[one_speed], cbm = cb * tab.mult[one_speed];
+                            k = one_speed * KT +
+                                draw_heading_lb<KT>(tab, lb_step_d(tab, s2, (x - gx) * im, (y - gy) * im, cbm), cbm,
+                                                    word);
+                        } else if (lb) {
+                            k = draw_multi_lb<KT>(tab, speed_on, x, y, gx, gy, bt, cb, cw, word, settle);
+                        } else {
+                            k = draw_multi(tab, speed_on, K, x, y, gx, gy, bt, cb, cw, lb, word, settle);
+                        }
+                    } else {
+                        k = draw_multi(tab, speed_on, K, x, y, gx, gy, bt, cb, cw, lb, word, settle);
+                    }
                 } else {
-                    red_add(c.counts + (size_t)(t - 1) * plane + key, (uint32_t)__popc(peers));
-                    if (c.flags) c.flags[(size_t)(t - 1) * c.fplane + fkey] = 1u; // idempotent
+                    k = draw<KT, FULL>(tab, enabled, s2, x, y, gx, gy, cb, lb, word);
                 }
             }
-        }
+            if constexpr (MS) {
+                // a draw too close to a CDF boundary for FP32 is settled in
+                // double-float by the whole warp, one flagged lane at a time
+                unsigned need = __ballot_sync(0xffffffffu, settle);
+                while (need) {
+                    const int src = __ffs((int)need) - 1;
+                    const int u = settle_multi_warp(tab, speed_on, K, x, y, gx, gy, bt, word, k, src);
+                    if (lane == src) k = u;
+                    need &= need - 1u;
+                }
+            }
+            advance(t, act ? k : 0);
+            flush(t); // at once: its registers are wanted by the next draw
+            done = t++;
+        } while (t <= c.T && (!FAST || !wfast || (near && ((t - 1) & 7) != 0)));
     }
+    if (done < c.T) flush(c.T);
 }
 
 } // namespace pm

@@ -1,0 +1,98 @@
+"""The closed-form heading draw against the weight-by-weight draw.
+
+A model with more than 16 beta values takes the weight-by-weight draw at every
+step. Padding a smaller model's beta grid to 17 values whose added components
+have a log-belief of -inf leaves every random choice as it is, so the two calls
+must agree in every count: no tolerance.
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2603_01122_gb300 as pm
+
+pytestmark = pytest.mark.gpu
+
+
+def _predict(K, speeds, speed_off, goals, beta, log_b, dt, N, T, W, H, res, z0, traced):
+    ctx = pm.pm_create(0)
+    try:
+        g, b = torch.tensor(goals).cuda(), torch.tensor(beta).cuda()
+        model = pm.make_model(K, 1.0, dt, g, b, speeds=speeds, speed_off=speed_off)
+        lb = torch.tensor(log_b).cuda()
+        counts = torch.empty((T, H, W), dtype=torch.int32, device="cuda")
+        oob = torch.empty(T, dtype=torch.int32, device="cuda")
+        grid = pm.make_grid(z0[0] - 0.5 * W * res, z0[1] - 0.5 * H * res, res, W, H)
+        if traced:
+            states = torch.empty((N, T, 2), device="cuda")
+            pm.pm_predict_occupancy_traced(ctx, model, lb, *z0, N, T, grid, 7, 3, counts, oob, N, states, None, None)
+        else:
+            pm.pm_predict_occupancy(ctx, model, lb, *z0, N, T, grid, 7, 3, counts, oob)
+        pm.pm_sync_status(ctx)
+        out = [counts.cpu().numpy(), oob.cpu().numpy()]
+        return out + [states.cpu().numpy()] if traced else out
+    finally:
+        pm.pm_destroy(ctx)
+
+
+@pytest.mark.parametrize("K,speeds,off,dt,b_lo,b_hi,near", [
+    (20, None, 0, 0.02, -2.0, 2.0, False),   # the fewest headings
+    (23, None, 0, 0.05, -2.0, 1.0, False),   # odd, not a template size
+    (36, None, 0, 0.02, -2.0, 2.0, True),    # goals reached: both forms in turn
+    (64, None, 0, 0.1, -2.0, 1.0, True),
+    (36, None, 0, 0.1, -2.0, 2.0, False),    # some rows beyond the usable kappa
+    (16, (0.5, 1.0), 0, 0.04, -1.0, 1.0, False),
+    (32, (0.5, 1.0, 1.5), 0, 0.02, -2.0, 2.0, True),
+    (20, (0.25, 1.0, 1.5, 2.0), 0b0101, 0.04, -1.0, 1.0, False),
+    (36, (0.5, 1.0), 0b10, 0.04, -2.0, 1.0, False),  # one speed left
+])
+@pytest.mark.parametrize("traced", [False, True])
+def test_equals_weight_by_weight(K, speeds, off, dt, b_lo, b_hi, near, traced):
+    rng = np.random.default_rng(K)
+    G, B, N, T, W, H, res, z0 = 3, 16, 3001, 61, 83, 77, 0.07, (1.5, -0.5)
+    goals = (np.array(z0) + rng.uniform(-1.0, 1.0, (G, 2)) * (0.5 if near else 8.0)).astype(np.float32)
+    beta = (10.0 ** np.linspace(b_lo, b_hi, B)).astype(np.float32)
+    beta[3] = -beta[3]  # a pedestrian walking away from the goal
+    beta[5] = 0.0
+    log_b = np.log(rng.dirichlet(np.ones(G * B))).astype(np.float32)
+    wide = np.full((G, B + 1), -np.inf, np.float32)
+    wide[:, :B] = log_b.reshape(G, B)
+    args = (dt, N, T, W, H, res, z0, traced)
+    got = _predict(K, speeds, off, goals, beta, log_b, *args)
+    want = _predict(K, speeds, off, goals, np.append(beta, np.float32(1.0)), wide.ravel(), *args)
+    assert got[0].sum() + got[1].sum() == N * T
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("K,speeds", [(36, None), (20, None), (64, None), (32, (0.5, 1.0, 1.5))])
+@pytest.mark.parametrize("marks", [0, 1])
+def test_batch_equals_weight_by_weight(K, speeds, marks):
+    rng = np.random.default_rng(K + 1)
+    n, B, T, W, H = 5, 9, 40, 61, 67
+    outs = []
+    goals = [torch.tensor(rng.uniform(-4.0, 4.0, (1 + i % 3, 2)).astype(np.float32)).cuda() for i in range(n)]
+    beta = (10.0 ** np.linspace(-2.0, 2.0, B)).astype(np.float32)
+    belief = [np.log(rng.dirichlet(np.ones(len(g) * B))).astype(np.float32).reshape(len(g), B) for g in goals]
+    for pad in (0, 17 - B):
+        ctx = pm.pm_create(0)
+        try:
+            b = torch.tensor(np.append(beta, np.ones(pad, np.float32))).cuda()
+            model = pm.make_model(K, 1.0, 0.03, goals[0], b, speeds=speeds)
+            batch = pm.pm_batch_create(ctx, model, n)
+            z0 = torch.zeros((n, 2), device="cuda")
+            lb = [torch.tensor(np.pad(p, ((0, 0), (0, pad)), constant_values=-np.inf).ravel()).cuda() for p in belief]
+            counts = torch.empty((n, T, H, W), dtype=torch.int32, device="cuda")
+            oob = torch.empty((n, T), dtype=torch.int32, device="cuda")
+            grid = pm.make_grid(-2.0, -2.0, 0.06, W, H)
+            if marks:
+                pm.pm_batch_set_block_flags(batch, 1)
+            pm.pm_batch_set(batch, [pm.make_human(goals[i], b, lb[i], z0[i], 500 + 333 * i, T, grid, 7, i, counts[i],
+                                                  oob[i]) for i in range(n)])
+            pm.pm_batch_predict(batch)
+            pm.pm_sync_status(ctx)
+            outs.append((counts.cpu().numpy(), oob.cpu().numpy()))
+            pm.pm_batch_destroy(batch)
+        finally:
+            pm.pm_destroy(ctx)
+    assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
