@@ -550,6 +550,8 @@ cudaError_t launch_adjoint(const AdjointArgs &a, cudaStream_t s)
                  : adjoint_kernel<8><<<grid, kAdjThreads, 0, s>>>(a); break;
     case 16: full ? adjoint_kernel<16, false, true><<<grid, kAdjThreads, 0, s>>>(a)
                   : adjoint_kernel<16><<<grid, kAdjThreads, 0, s>>>(a); break;
+    case 24: full ? adjoint_kernel<24, false, true><<<grid, kAdjThreads, 0, s>>>(a)
+                  : adjoint_kernel<24><<<grid, kAdjThreads, 0, s>>>(a); break;
     case 36: full ? adjoint_kernel<36, false, true><<<grid, kAdjThreads, 0, s>>>(a)
                   : adjoint_kernel<36><<<grid, kAdjThreads, 0, s>>>(a); break;
     default: full ? adjoint_kernel<64, false, true><<<grid, kAdjThreads, 0, s>>>(a)

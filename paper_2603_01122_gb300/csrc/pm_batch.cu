@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 3) batch_rollout_kernel(cons
     __shared__ float s_z0[2];
     extern __shared__ __align__(16) uint32_t dyn[];
     const int tid = threadIdx.x, nthr = blockDim.x;
-    for (int k = tid; k < KT; k += nthr) sh.step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
+    for (int k = tid; k < step_entries(KT); k += nthr) sh.step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
     const int n_items = *a.n_items;
     int cur = -1;
     for (;;) {
@@ -158,7 +158,7 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
         for (int u = tid; u < a.tab.S * a.K; u += blockDim.x)
             step[u] = make_float2(a.tab.msx[u / a.K][u % a.K], a.tab.msy[u / a.K][u % a.K]);
     } else {
-        for (int k = tid; k < KT; k += blockDim.x) step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
+        for (int k = tid; k < step_entries(KT); k += blockDim.x) step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
     }
     __syncthreads();
     char *slab = reinterpret_cast<char *>(dyn) + (size_t)warp * (MS ? kWarpTableBytesMS : kWarpTableBytes);
@@ -526,6 +526,7 @@ cudaError_t batch_dispatch(const BatchArgs &a, const RolloutShape &sh, int block
     switch (KT) {
     case 8: return full ? batch_shape<8, true>(a, sh, blocks, dyn, s, occ) : batch_shape<8, false>(a, sh, blocks, dyn, s, occ);
     case 16: return full ? batch_shape<16, true>(a, sh, blocks, dyn, s, occ) : batch_shape<16, false>(a, sh, blocks, dyn, s, occ);
+    case 24: return batch_shape<24, false>(a, sh, blocks, dyn, s, occ); // no FULL form
     case 36: return full ? batch_shape<36, true>(a, sh, blocks, dyn, s, occ) : batch_shape<36, false>(a, sh, blocks, dyn, s, occ);
     default: return full ? batch_shape<64, true>(a, sh, blocks, dyn, s, occ) : batch_shape<64, false>(a, sh, blocks, dyn, s, occ);
     }

@@ -227,7 +227,7 @@ constexpr int kFlagShift = 4, kFlagBlock = 1 << kFlagShift;
 // Rollout launch (defined next to its kernels).
 // `head` is a zeroed device counter of 32-particle chunks.
 cudaError_t launch_rollout(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s);
-int rollout_kt_for(int K); // template bucket for K (8, 16, 36 or 64)
+int rollout_kt_for(int K); // template bucket for K (8, 16, 24, 36 or 64)
 size_t rollout_static_smem_estimate();
 
 } // namespace pm

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, (FAST && KT == 64) ? 5 : kWar
         comp[j] = make_float4(cbj, a.goals[2 * g], a.goals[2 * g + 1], lb_flag(a.tab, cbj));
         if (bad_component(cbj, comp[j].y, comp[j].z)) flag_status(a.status, kStatusModel);
     }
-    for (int k = tid; k < KT; k += blockDim.x) step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
+    for (int k = tid; k < step_entries(KT); k += blockDim.x) step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
     if (tid < 32 && belief_cdf(a.log_b, J, cdf, tid) && tid == 0) flag_status(a.status, kStatusBelief);
     __syncthreads();
 
@@ -199,14 +199,17 @@ template <int KT, bool TRACE>
 cudaError_t launch_kt(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
     // every heading enabled and K == KT: the FULL form, in closed form where
-    // K >= kFastMinK
+    // K >= kFastMinK; the bucket of 24 has no FULL form (its weight-by-weight
+    // draw is the general one, as in the bucket of 36 before it)
     const bool fast = fast_applies(a.K, a.enabled, 1);
     auto k = rollout_warp_kernel<KT, false, false, TRACE>;
     if constexpr (KT >= kFastMinK) {
         if (fast) k = rollout_warp_kernel<KT, false, true, TRACE>;
     }
-    const uint64_t all = (KT >= 64) ? ~0ull : ((1ull << KT) - 1ull);
-    if (a.K == KT && (a.enabled & all) == all) k = rollout_warp_kernel<KT, true, (KT >= kFastMinK), TRACE>;
+    if constexpr (KT != 24) {
+        const uint64_t all = (KT >= 64) ? ~0ull : ((1ull << KT) - 1ull);
+        if (a.K == KT && (a.enabled & all) == all) k = rollout_warp_kernel<KT, true, (KT >= kFastMinK), TRACE>;
+    }
     int n = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kWarpCtaThreads, 0);
     if (e != cudaSuccess) return e;
@@ -237,6 +240,7 @@ cudaError_t dispatch(const RolloutArgs &a, unsigned *head, int sm_count, cudaStr
     switch (rollout_kt_for(a.K)) {
     case 8: return launch_kt<8, TRACE>(a, head, sm_count, s, occ);
     case 16: return launch_kt<16, TRACE>(a, head, sm_count, s, occ);
+    case 24: return launch_kt<24, TRACE>(a, head, sm_count, s, occ);
     case 36: return launch_kt<36, TRACE>(a, head, sm_count, s, occ);
     default: return launch_kt<64, TRACE>(a, head, sm_count, s, occ);
     }
@@ -248,6 +252,7 @@ int rollout_kt_for(int K)
 {
     if (K <= 8) return 8;
     if (K <= 16) return 16;
+    if (K <= 24) return 24;
     if (K <= 36) return 36;
     return 64;
 }

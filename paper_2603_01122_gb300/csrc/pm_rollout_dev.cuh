@@ -146,15 +146,24 @@ __device__ __forceinline__ int draw_heading(const HeadingTab &tab, uint64_t enab
         }
         return sel0 + sel1;
     } else {
+        // (the same packed pairs as above; a disabled heading's weight is 0)
+        static_assert(KT % 2 == 0, "pairs of headings");
+        const f32x2 DX = f2_pack(dx, dx), DY = f2_pack(dy, dy);
+        const f32x2 DD = f2_pack(D, D), NDD = f2_pack(-D, -D), HD = f2_pack(hD, hD), C3 = f2_pack(c3, c3);
+        const f32x2 *TX = reinterpret_cast<const f32x2 *>(tab.tx);
+        const f32x2 *TY = reinterpret_cast<const f32x2 *>(tab.ty);
         float dv[KT];
-        float dref = 0.0f;
+        f32x2 DREF = 0ull;
 #pragma unroll
-        for (int k = 0; k < KT; ++k) {
-            const float p = fmaf(tab.tx[k], dx, tab.ty[k] * dy);
-            const float dk = sqrt_approx(fmaxf(D + p, 0.0f));
-            const float rk = fmaf(-dk, dk, D) + p;
-            if (k == 0) dref = dk;
-            dv[k] = fmaf(rk, fmaf(p, c3, hD), dk - dref);
+        for (int q = 0; q < KT / 2; ++q) {
+            const f32x2 P = f2_fma(TX[q], DX, f2_mul(TY[q], DY));
+            float x0, x1;
+            f2_unpack(f2_add(DD, P), x0, x1);
+            const float d0 = sqrt_approx(fmaxf(x0, 0.0f)), d1 = sqrt_approx(fmaxf(x1, 0.0f));
+            const f32x2 DK = f2_pack(d0, d1);
+            if (q == 0) DREF = f2_pack(d0, d0);
+            const f32x2 R = f2_sub(P, f2_fma(DK, DK, NDD));
+            f2_unpack(f2_fma(R, f2_fma(P, C3, HD), f2_sub(DK, DREF)), dv[2 * q], dv[2 * q + 1]);
         }
         // the most probable heading: the nearest for beta >= 0, the farthest
         // for beta < 0, so that every exponent below is <= 0
@@ -163,16 +172,20 @@ __device__ __forceinline__ int draw_heading(const HeadingTab &tab, uint64_t enab
         for (int k = 0; k < KT; ++k)
             if (FULL || ((enabled >> k) & 1ull)) dext = (cb >= 0.0f) ? fminf(dext, dv[k]) : fmaxf(dext, dv[k]);
         const float base = __fmul_rd(dext, cb); // rounded down: every exponent below is <= 0
-        const float nc = -cb;
+        const f32x2 NC = f2_pack(-cb, -cb), BASE = f2_pack(base, base);
+        const f32x2 SC = f2_pack(kWScale, kWScale), MG = f2_pack(kWMagic, kWMagic);
         uint32_t C[KT];
         uint32_t S = 0;
 #pragma unroll
-        for (int k = 0; k < KT; ++k) {
-            const float e = ex2_approx(fmaf(dv[k], nc, base));
-            uint32_t E = __float_as_uint(fmaf(e, kWScale, kWMagic)) - kWBits;
-            if (!FULL && !((enabled >> k) & 1ull)) E = 0u;
-            S += E;
-            C[k] = S;
+        for (int q = 0; q < KT / 2; ++q) {
+            float a0, a1, w0, w1;
+            f2_unpack(f2_fma(f2_pack(dv[2 * q], dv[2 * q + 1]), NC, BASE), a0, a1);
+            f2_unpack(f2_fma(f2_pack(ex2_approx(a0), ex2_approx(a1)), SC, MG), w0, w1);
+            const uint32_t E0 = __float_as_uint(w0) - kWBits, E1 = __float_as_uint(w1) - kWBits;
+            S += ((enabled >> (2 * q)) & 1ull) ? E0 : 0u;
+            C[2 * q] = S;
+            S += ((enabled >> (2 * q + 1)) & 1ull) ? E1 : 0u;
+            C[2 * q + 1] = S;
         }
         const uint32_t thr = (uint32_t)(((uint64_t)(word >> 8) * (uint64_t)S) >> 24);
         int sel = 0;
@@ -354,6 +367,10 @@ __device__ __forceinline__ float lb_flag(const HeadingTab &tab, float cb)
 // A component's table entry must be finite (goal and beta w2 log2(e)).
 __device__ __forceinline__ bool bad_component(float cb, float gx, float gy) { return !isfinite(cb + gx + gy); }
 
+// Entries of the step table that a draw of the bucket KT may name (beyond the
+// K headings they are zero: an unusable model leaves its particles in place).
+__host__ __device__ constexpr int step_entries(int KT) { return KT == 24 ? 36 : KT; }
+
 // The heading draw of one particle: the fused bound form where it applies.
 template <int KT, bool FULL>
 __device__ __forceinline__ int draw(const HeadingTab &tab, uint64_t enabled, float s2, float x, float y, float gx,
@@ -368,7 +385,7 @@ __device__ __forceinline__ int draw(const HeadingTab &tab, uint64_t enabled, flo
     }
     // k < K whenever the total weight S > 0, which finite inputs guarantee;
     // the clamp keeps the step-table read in bounds for any input
-    return min(k, KT - 1);
+    return min(k, step_entries(KT) - 1);
 }
 
 // ---------------------------------------------------------------------------
