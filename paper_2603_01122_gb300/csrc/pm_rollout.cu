@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, (FAST && KT == 64) ? 5 : kWar
     __shared__ uint32_t words[kWarpCtaThreads / 32 * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31;
     const int J = a.G * a.B;
+    pdl_wait(); // the belief, the zeroed outputs and the rows
     for (int j = tid; j < J; j += blockDim.x) {
         const int g = j / a.B, b = j - g * a.B;
         const float cbj = a.beta[b] * a.w2_log2e;
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     __shared__ uint32_t words[kWarpCtaThreads / 32 * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31;
     const int J = a.G * a.B;
+    pdl_wait(); // the belief, the zeroed outputs and the rows
     for (int j = tid; j < J; j += blockDim.x) {
         const int g = j / a.B, b = j - g * a.B;
         const float cbj = a.beta[b] * a.w2_log2e;
@@ -191,8 +193,7 @@ cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cud
     int64_t blocks = (int64_t)sm_count * (n > 0 ? n : 1);
     if (need < blocks) blocks = need;
     cudaGetLastError();
-    rollout_multi_kernel<KT, TRACE><<<(unsigned)blocks, kWarpCtaThreads, 0, s>>>(a, head);
-    return cudaGetLastError();
+    return launch_early(rollout_multi_kernel<KT, TRACE>, (unsigned)blocks, kWarpCtaThreads, s, a, head);
 }
 
 template <int KT, bool TRACE>
@@ -222,8 +223,7 @@ cudaError_t launch_kt(const RolloutArgs &a, unsigned *head, int sm_count, cudaSt
     int64_t blocks = (int64_t)sm_count * (n > 0 ? n : 1);
     if (need < blocks) blocks = need;
     cudaGetLastError(); // clear errors of earlier calls whose failure was handled
-    k<<<(unsigned)blocks, kWarpCtaThreads, 0, s>>>(a, head);
-    return cudaGetLastError();
+    return launch_early(k, (unsigned)blocks, kWarpCtaThreads, s, a, head);
 }
 
 template <bool TRACE>
