@@ -109,3 +109,18 @@ def test_mppi_rejects_bad_parameters(ctx):
         with pytest.raises(pm.PmError) as e:
             pm.pm_mppi_solve(ctx, params, z0, dev(u_ref), dev(delta), None, 0, None, ctg, u_opt)
         assert e.value.status == pm.PM_EINVAL
+
+
+@pytest.mark.parametrize("N,T,stride", [(65, 90, 1), (64, 91, 2), (1024, 6, 3), (1023, 7, 40), (2, 1, 1)])
+def test_mppi_rollout_forms(ctx, N, T, stride):
+    """Both rollout kernels (the line lies at 90 steps), at the edges of their
+    CTAs and look-ahead. Same bound as above, on the costs away from cell edges;
+    past the prediction's end (large stride) no collision is charged."""
+    p, z0, u_ref, delta, prob, grid = _scenario(N, T, N + T)
+    p["pred_stride"] = stride
+    S_gpu, u_gpu = _gpu(ctx, p, z0, u_ref, delta, prob, grid)
+    _, _, S, edge = M.solve(p, np.float32(z0).astype(np.float64), u_ref, delta, prob, grid)
+    ok = np.abs(S_gpu - S) <= 1e-4 * (1.0 + S)
+    assert np.all(ok[:, edge >= 1e-3])
+    dmax = np.abs(delta).max()
+    assert np.all(np.abs(u_gpu - M.update(u_ref, delta, S_gpu, p["temperature"])) <= 1e-5 * dmax + 1e-7)
