@@ -487,10 +487,18 @@ pm_status posterior_impl(pm_ctx *ctx, const pm_model *model, const float *obs_xy
     a.log_prior = log_prior;
     a.log_b = log_belief;
     const int n_chunks = pm::posterior_chunks(n_obs, &a.steps_per_chunk);
-    st = ensure_posterior_scratch(ctx, pm::posterior_scratch_bytes(n_chunks, model->G * model->B));
+    // the partial sums, then (at an 8-byte boundary) the groups' folded components
+    const size_t part = (pm::posterior_scratch_bytes(n_chunks, model->G * model->B) + 7) & ~(size_t)7;
+    st = ensure_posterior_scratch(ctx, part + J * sizeof(float2));
     if (st != PM_OK) return st;
     a.part = (float *)ctx->post_scratch;
     a.ticket = ctx->ticket;
+    // a warp per component and chunk: beyond 32 components several CTAs share
+    // a chunk (256 components, 200 steps: 85 us with 32 warps a chunk,
+    // 32 us with eight times as many)
+    a.groups = (int)((J + 31) / 32);
+    a.fold = (float2 *)((char *)ctx->post_scratch + part);
+    a.gticket = ctx->ticket + 16;
     a.status = status_word(ctx);
     cudaError_t e = pm::launch_posterior(a, n_chunks, stream);
     if (e != cudaSuccess) return cuda_fail(e, "posterior launch");

@@ -55,7 +55,12 @@ struct PosteriorArgs {
     float *part;         // scratch: per (chunk, component) accumulators
     unsigned *ticket;    // scratch: chunks finished so far (0 between calls)
     unsigned *status;    // context status word (or NULL)
+    // several groups of components (a CTA per chunk and group; 0: one group)
+    int groups;
+    float2 *fold;        // scratch [J]: a component's unnormalised log-belief
+    unsigned *gticket;   // kMaxPostGroups chunk tickets, then "a step moved the belief" (0 between calls)
 };
+constexpr int kMaxPostGroups = kMaxJ / 32;
 
 // Arguments of the log-likelihood / adjoint kernel.
 struct AdjointArgs {
@@ -138,7 +143,7 @@ struct SmoothSrc {
 };
 
 struct SmoothArgs {
-    const SmoothSrc *srcs; // device source records, or nullptr: `single`
+    const SmoothSrc *srcs; // device source records, or nullptr: `single`, on the output grid
     const int *n_srcs;     // device: number of records
     SmoothSrc single;
     float w[2 * kMaxSmoothR + 1]; // normalised taps w_{-R..R}

@@ -169,14 +169,18 @@ __device__ __forceinline__ void step_loglik_ms(const SpeedSet &sp, const float4 
 
 // One chunk of one human's observed steps; the last chunk of the human to
 // finish folds all chunks and writes the posterior. MS: several speeds.
-template <bool MS>
-__device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const PostHuman &h, int chunk, int nchunk)
+// GROUPS: the CTA takes the components of group `grp` of a.groups; the last
+// chunk of a group folds the group, and the last group to be folded normalises.
+template <bool MS, bool GROUPS>
+__device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const PostHuman &h, int chunk, int nchunk,
+                                                int grp)
 {
     __shared__ int last;
     __shared__ float2 su[kMaxK]; // unit heading vectors
     __shared__ float4 cu[MS ? kMsPerLane * 32 : 1]; // several speeds: (e_k, sl_q, enabled) of control u
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int J = h.G * h.B;
+    const int j0 = GROUPS ? grp * nwarp + warp : warp, jstep = GROUPS ? a.groups * nwarp : nwarp;
     const int t0 = chunk * h.steps_per_chunk;
     const int t1 = min(h.n_obs, t0 + h.steps_per_chunk);
     // the table goes through shared memory once per CTA: lanes reading
@@ -198,7 +202,7 @@ __device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const Po
     const float ux0 = on0 ? su[k0].x : 0.0f, uy0 = on0 ? su[k0].y : 0.0f;
     const float ux1 = on1 ? su[k1].x : 0.0f, uy1 = on1 ? su[k1].y : 0.0f;
 
-    for (int j = warp; j < J; j += nwarp) {
+    for (int j = j0; j < J; j += jstep) {
         const int g = j / h.B, b = j - g * h.B;
         const float bw = h.beta[b] * a.w2;
         const float gx = h.goals[2 * g], gy = h.goals[2 * g + 1];
@@ -250,7 +254,8 @@ __device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const Po
 
     // the last chunk to finish combines and normalises
     __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(h.ticket, 1u) == (unsigned)(nchunk - 1));
+    unsigned *ticket = GROUPS ? a.gticket + grp : h.ticket;
+    if (threadIdx.x == 0) last = (atomicAdd(ticket, 1u) == (unsigned)(nchunk - 1));
     __syncthreads();
     if (!last) return;
     __threadfence();
@@ -266,7 +271,7 @@ __device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const Po
     __shared__ int moved;
     if (threadIdx.x == 0) moved = 0;
     __syncthreads();
-    for (int j = warp; j < J; j += nwarp) {
+    for (int j = j0; j < J; j += jstep) {
         Acc acc;
         acc_init(acc);
         for (int c = lane; c < nchunk; c += 32) {
@@ -308,6 +313,22 @@ __device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const Po
         }
     }
     __syncthreads();
+    if constexpr (GROUPS) {
+        // this group's components to scratch; the last group reads them all
+        for (int j = j0; j < J; j += jstep)
+            if (lane == 0) a.fold[j] = L[j];
+        if (threadIdx.x == 0) *ticket = 0u;
+        if (threadIdx.x == 0 && moved) atomicOr(a.gticket + kMaxPostGroups, 1u);
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = (atomicAdd(h.ticket, 1u) == (unsigned)(a.groups - 1));
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        for (int j = threadIdx.x; j < J; j += blockDim.x) L[j] = __ldcg(a.fold + j);
+        if (threadIdx.x == 0) moved = (int)atomicExch(a.gticket + kMaxPostGroups, 0u);
+        __syncthreads();
+    }
     if (warp == 0 && !moved) {
         for (int j = lane; j < J; j += 32) h.log_b[j] = h.log_prior[j];
         if (lane == 0) *h.ticket = 0u;
@@ -329,7 +350,7 @@ __device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const Po
 // MS: several speeds. A template parameter rather than a branch, so that a
 // launch carries only its own form's code (the kernel runs once per call on
 // a cold instruction cache).
-template <bool MS>
+template <bool MS, bool GROUPS>
 __global__ void __launch_bounds__(1024) posterior_kernel(const __grid_constant__ PosteriorArgs a)
 {
     pdl_release(); // what prepares the rollout may start beside this grid
@@ -346,7 +367,7 @@ __global__ void __launch_bounds__(1024) posterior_kernel(const __grid_constant__
     h.part = a.part;
     h.ticket = a.ticket;
     h.speed_on = a.sp.speed_on;
-    posterior_chunk<MS>(a, h, blockIdx.x, gridDim.x);
+    posterior_chunk<MS, GROUPS>(a, h, blockIdx.x, gridDim.x, blockIdx.y);
 }
 
 // Batched form: blockIdx.y is the human; the CTAs of a row stride over its
@@ -361,7 +382,7 @@ __global__ void __launch_bounds__(1024) posterior_batch_kernel(const __grid_cons
     if (h.n_obs <= 0 || h.log_b == nullptr || h.log_prior == nullptr) return;
     const int nchunk = (h.n_obs + h.steps_per_chunk - 1) / h.steps_per_chunk;
     for (int ch = blockIdx.x; ch < nchunk; ch += gridDim.x) {
-        posterior_chunk<MS>(a, h, ch, nchunk);
+        posterior_chunk<MS, false>(a, h, ch, nchunk, 0);
     }
 }
 
@@ -396,8 +417,15 @@ cudaError_t launch_posterior(const PosteriorArgs &a, int n_chunks, cudaStream_t 
     const int J = a.G * a.B;
     int threads = 32 * J;
     if (threads > 1024) threads = 1024;
-    if (a.sp.S > 0) posterior_kernel<true><<<n_chunks, threads, 0, s>>>(a);
-    else posterior_kernel<false><<<n_chunks, threads, 0, s>>>(a);
+    if (a.groups > 1) {
+        const dim3 grid(n_chunks, a.groups);
+        if (a.sp.S > 0) posterior_kernel<true, true><<<grid, threads, 0, s>>>(a);
+        else posterior_kernel<false, true><<<grid, threads, 0, s>>>(a);
+    } else if (a.sp.S > 0) {
+        posterior_kernel<true, false><<<n_chunks, threads, 0, s>>>(a);
+    } else {
+        posterior_kernel<false, false><<<n_chunks, threads, 0, s>>>(a);
+    }
     return cudaGetLastError();
 }
 
