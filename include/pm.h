@@ -425,6 +425,13 @@ pm_status pm_loglik_backward(pm_ctx *ctx, const pm_model *model, int32_t M, cons
                              float grad_out, float *loglik, float *d_goals, float *d_speed,
                              float *d_w, void *stream);
 
+/* L and its unscaled gradient [2G+3] in FP64 (device): d_goals [G][2], d_speed,
+ * d_w1, d_w2, from one pass; scaled and rounded to FP32 it is what
+ * pm_loglik_backward returns. */
+pm_status pm_loglik_value_grad(pm_ctx *ctx, const pm_model *model, int32_t M, const int32_t *offsets,
+                               int32_t n_points, const float *traj_xy, const float *log_prior,
+                               float *loglik, double *grad, void *stream);
+
 /* ---- for callers that cannot allocate ------------------------------------- */
 
 /* The paper has no counterpart to this call; it serves callers that must not

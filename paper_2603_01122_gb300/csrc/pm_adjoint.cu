@@ -496,6 +496,8 @@ __global__ void __launch_bounds__(kAdjThreads) adjoint_kernel(const __grid_const
         if (lane == 0) {
             if (q == 0) {
                 *a.loglik = (float)s;
+            } else if (a.grad64) {
+                a.grad64[q - 1] = s;
             } else if (q <= 2 * a.G) {
                 a.d_goals[q - 1] = (float)(s * (double)a.grad_out);
             } else if (q == 2 * a.G + 1) {

@@ -507,7 +507,7 @@ pm_status posterior_impl(pm_ctx *ctx, const pm_model *model, const float *obs_xy
 
 pm_status loglik_impl(pm_ctx *ctx, const pm_model *model, int32_t M, const int32_t *offsets, int32_t n_points,
                       const float *traj_xy, const float *log_prior, bool want_grad, float grad_out, float *loglik,
-                      float *d_goals, float *d_speed, float *d_w, cudaStream_t stream)
+                      float *d_goals, float *d_speed, float *d_w, cudaStream_t stream, double *grad64 = nullptr)
 {
     if (!ctx) return fail(PM_EINVAL, "ctx is NULL");
     pm_status st = check_model(model);
@@ -515,7 +515,7 @@ pm_status loglik_impl(pm_ctx *ctx, const pm_model *model, int32_t M, const int32
     if (M < 1) return fail(PM_EINVAL, "M=%d must be >= 1", M);
     if (n_points < 0) return fail(PM_EINVAL, "n_points must be >= 0");
     if (!offsets || !traj_xy || !log_prior || !loglik) return fail(PM_EINVAL, "a device pointer is NULL");
-    if (want_grad && (!d_goals || !d_speed || !d_w)) return fail(PM_EINVAL, "gradient outputs are NULL");
+    if (want_grad && !grad64 && (!d_goals || !d_speed || !d_w)) return fail(PM_EINVAL, "gradient outputs are NULL");
     if (!std::isfinite(grad_out)) return fail(PM_EINVAL, "grad_out must be finite");
     DeviceScope dev(ctx->device);
     st = ensure_posterior_scratch(ctx, 0); // allocates the ticket word
@@ -566,6 +566,7 @@ pm_status loglik_impl(pm_ctx *ctx, const pm_model *model, int32_t M, const int32
     a.ticket = ctx->ticket + 1; // its own word of the ticket block
     a.status = status_word(ctx);
     a.loglik = loglik;
+    a.grad64 = grad64;
     a.d_goals = d_goals;
     a.d_speed = d_speed;
     a.d_w = d_w;
@@ -1553,6 +1554,16 @@ pm_status pm_loglik_forward(pm_ctx *ctx, const pm_model *model, int32_t M, const
     PM_RANGE("pm_loglik_forward");
     return loglik_impl(ctx, model, M, offsets, n_points, traj_xy, log_prior, false, 1.0f, loglik, nullptr,
                        nullptr, nullptr, (cudaStream_t)stream);
+}
+
+pm_status pm_loglik_value_grad(pm_ctx *ctx, const pm_model *model, int32_t M, const int32_t *offsets,
+                               int32_t n_points, const float *traj_xy, const float *log_prior, float *loglik,
+                               double *grad, void *stream)
+{
+    PM_RANGE("pm_loglik_value_grad");
+    if (!grad) return fail(PM_EINVAL, "grad is NULL");
+    return loglik_impl(ctx, model, M, offsets, n_points, traj_xy, log_prior, true, 1.0f, loglik, nullptr, nullptr,
+                       nullptr, (cudaStream_t)stream, grad);
 }
 
 pm_status pm_loglik_backward(pm_ctx *ctx, const pm_model *model, int32_t M, const int32_t *offsets,

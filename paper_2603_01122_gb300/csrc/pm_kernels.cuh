@@ -86,6 +86,7 @@ struct AdjointArgs {
     unsigned *ticket;      // scratch ticket (0 between calls)
     unsigned *status;      // context status word (or NULL)
     float *loglik;
+    double *grad64;        // unscaled gradient [2G+3] (goals, v, w1, w2) instead of the three below, or NULL
     float *d_goals;
     float *d_speed;
     float *d_w;
