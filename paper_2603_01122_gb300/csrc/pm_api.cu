@@ -279,7 +279,7 @@ void fill_rollout_tables(const pm_model *m, pm::RolloutArgs &a)
     a.fc.cK = (float)std::cos(half);
     a.fc.sK = (float)std::sin(half);
     a.fc.K2pi = (float)(0.5 / half);
-    a.fc.K = (float)m->K;
+    a.fc.K = m->K;
 }
 
 // What builds the closed-form draw's rows at `rows`; rows == NULL (nothing to

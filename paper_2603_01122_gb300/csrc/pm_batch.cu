@@ -581,7 +581,7 @@ cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, i
     const unsigned rows = fp.rows ? (fp.B * fp.S + kRowsPerCta - 1) / kRowsPerCta : 0;
     if (blocks + rows == 0) return cudaSuccess;
     cudaGetLastError(); // clear errors of earlier calls whose failure was handled
-    return launch_early(zero_outputs_kernel, (unsigned)blocks + rows, kRowThreads, s, counts, words, oob, T, head,
+    return launch_early(zero_outputs_kernel, (unsigned)blocks + rows, kRowThreads, 0, s, counts, words, oob, T, head,
                         (int)blocks, fp);
 }
 

@@ -43,6 +43,7 @@ struct __align__(16) FastRow {
     float a0[kFastD];        // mean weight over the headings, times the speed's factor exp(-beta w1 v dt (m - m_0))
     float kappa, rho_max, tol, s; // rho_max = -1: the row is not usable
     float2 guess[kFastGuess];     // F^-1 at 2 pi j / kFastGuess, and the step to the next
+    float pad[4]; // an odd number of 16-byte words: rows of different lanes lie in different banks
 };
 
 struct FastPrep {
@@ -331,8 +332,8 @@ __host__ __device__ __forceinline__ FastDraw fast_begin(const FastConst &fc, con
 }
 
 // One third-order step of the draw; the heading, or -1 where the solution is
-// too close to a boundary for tolx (a fraction of the running total) and the
-// step's own error.
+// too close to a boundary for tolx (K times a fraction of the running total) and
+// the step's own error.
 __host__ __device__ __forceinline__ int fast_step(const FastConst &fc, const F2 (&P)[kFastP], float rho, float kappa,
                                                   float tolx, FastDraw &w)
 {
@@ -357,9 +358,9 @@ __host__ __device__ __forceinline__ int fast_step(const FastConst &fc, const F2 
     const int k = fast_floor(x, kf);
     const float fr = x - kf;
     const float e = ak * dl2 * fmaf(ak + 0.5f, fabsf(w.dl), fmaf(2.0f, rho, 0.1f)); // error of the step
-    const float band = fmaf(tolx * fc.K, inv, e * fc.K2pi);
+    const float band = fmaf(tolx, inv, e * fc.K2pi);
     // inv > 0 holds wherever the fit is good; NaN anywhere fails the test
-    const bool ok = fminf(fr, 1.0f - fr) > band && inv > 0.0f && kf >= 0.0f && kf < fc.K;
+    const bool ok = fminf(fr, 1.0f - fr) > band && inv > 0.0f && (unsigned)k < (unsigned)fc.K;
     return ok ? k : -1;
 }
 

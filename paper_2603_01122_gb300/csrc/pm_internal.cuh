@@ -143,7 +143,8 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... Params, typename... Args>
-cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, cudaStream_t s, Args... args)
+cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t dyn, cudaStream_t s,
+                         Args... args)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -151,6 +152,7 @@ cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned th
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = dyn;
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
@@ -208,7 +210,7 @@ struct FastRow;
 struct FastConst {
     float cK, sK; // cos, sin of pi / K
     float K2pi;   // K / (2 pi)
-    float K;
+    int K;
 };
 
 // Arguments of the rollout kernel (Algorithm 1 + emplacement).

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     __shared__ float betas[kMaxJ];
     __shared__ uint32_t cdf[kMaxJ];
     __shared__ float2 step[PM_MAX_SPEEDS * kMaxK];
+    extern __shared__ float4 fast_sm[]; // the rows of the closed-form draw: a lane reads another one at each step
     __shared__ uint32_t words[kWarpCtaThreads / 32 * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31;
     const int J = a.G * a.B;
@@ -134,6 +135,9 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
         if (bad_component(cbj, comp[j].y, comp[j].z)) flag_status(a.status, kStatusModel);
         betas[j] = a.beta[b];
     }
+    if (a.fast)
+        for (int i = tid; i < a.B * a.tab.S * (int)(sizeof(FastRow) / 16); i += blockDim.x)
+            fast_sm[i] = reinterpret_cast<const float4 *>(a.fast)[i];
     for (int u = tid; u < a.tab.S * a.K; u += blockDim.x)
         step[u] = make_float2(a.tab.msx[u / a.K][u % a.K], a.tab.msy[u / a.K][u % a.K]);
     if (tid < 32 && belief_cdf(a.log_b, J, cdf, tid) && tid == 0) flag_status(a.status, kStatusBelief);
@@ -162,7 +166,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     c.tr_states = a.tr_states;
     c.tr_head = a.tr_head;
     c.tr_comp = a.tr_comp;
-    c.fast = a.fast;
+    c.fast = a.fast ? reinterpret_cast<const FastRow *>(fast_sm) : nullptr;
     c.B = a.B;
     c.flags = nullptr;
     c.fbx = c.fplane = 0;
@@ -182,7 +186,11 @@ template <int KT, bool TRACE>
 cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
     int n = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rollout_multi_kernel<KT, TRACE>, kWarpCtaThreads, 0);
+    const size_t dyn = a.fast ? (size_t)a.B * a.tab.S * sizeof(FastRow) : 0;
+    cudaError_t e = cudaFuncSetAttribute(rollout_multi_kernel<KT, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kFastMaxB * PM_MAX_SPEEDS * sizeof(FastRow)));
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rollout_multi_kernel<KT, TRACE>, kWarpCtaThreads, dyn);
     if (e != cudaSuccess) return e;
     if (occ) {
         *occ = n;
@@ -193,7 +201,7 @@ cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cud
     int64_t blocks = (int64_t)sm_count * (n > 0 ? n : 1);
     if (need < blocks) blocks = need;
     cudaGetLastError();
-    return launch_early(rollout_multi_kernel<KT, TRACE>, (unsigned)blocks, kWarpCtaThreads, s, a, head);
+    return launch_early(rollout_multi_kernel<KT, TRACE>, (unsigned)blocks, kWarpCtaThreads, dyn, s, a, head);
 }
 
 template <int KT, bool TRACE>
@@ -223,7 +231,7 @@ cudaError_t launch_kt(const RolloutArgs &a, unsigned *head, int sm_count, cudaSt
     int64_t blocks = (int64_t)sm_count * (n > 0 ? n : 1);
     if (need < blocks) blocks = need;
     cudaGetLastError(); // clear errors of earlier calls whose failure was handled
-    return launch_early(k, (unsigned)blocks, kWarpCtaThreads, s, a, head);
+    return launch_early(k, (unsigned)blocks, kWarpCtaThreads, 0, s, a, head);
 }
 
 template <bool TRACE>

@@ -1187,12 +1187,12 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                     rmin = row->rho_max > 0.0f ? row->s / row->rho_max : INFINITY;
                     ftol_r = fabsf(row->kappa) / row->s;
                     fkap = row->kappa;
-                    ftol = row->tol;
+                    ftol = row->tol * (float)fc.K;
                 }
                 fr2 = rmin * rmin * 1.00001f;
                 // the weight-by-weight draw's exponents carry the rounding of
                 // beta w2 r: some 2^-24 of it after its residual correction
-                ftol_r *= 4e-10f;
+                ftol_r *= 4e-10f * (float)fc.K;
             }
         }
     }
@@ -1234,12 +1234,13 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
     // matched over the warp. The histogram add itself follows in flush(), at
     // the next step's first wait: match.any takes long to answer, and nothing
     // of the next draw depends on it. Idle lanes run along with their own key.
+    const uint32_t lower = act ? (1u << lane) - 1u : 0xFFFFFFFFu; // (an idle lane never leads)
     uint32_t pkey = 0u, ppeers = 0u;
     int pfkey = 0;
     auto flush = [&](int t) { // the adds of step t
         if (TRACE && !c.hist) return;
         // the lowest lane of each group of equal keys adds the group's size
-        if (pkey != 0xFFFFFFFFu && (ppeers & ((1u << lane) - 1u)) == 0u) {
+        if ((ppeers & lower) == 0u) {
             const bool in = pkey != 0xFFFFFFFEu;
             uint32_t *dst = in ? crow + pkey : c.oob + (t - 1);
             red_add(dst, (uint32_t)__popc(ppeers));
@@ -1281,7 +1282,8 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
         bool near = true; // several weight-by-weight steps follow
         int k = 0;
         if constexpr (FAST) {
-            if (wfast) {
+            const float dx0 = x - gx, dy0 = y - gy;
+            if (wfast && __all_sync(0xffffffffu, !act || fmaf(dx0, dx0, dy0 * dy0) > fr2)) {
                 // The closed-form steps, until one that the warp cannot take
                 // (a goal too close) or that some lanes leave open. The row's
                 // values live only in this loop: the weight-by-weight draw
@@ -1329,7 +1331,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                         base = sp * K;
                         rho = o->s * ri;
                         kap = o->kappa;
-                        tol = (2.0f * o->tol + far) * (total * iw); // (the mean weights carry the same error)
+                        tol = fmaf(2.0f * (float)fc.K, o->tol, far) * (total * iw); // (the mean weights carry the same error)
                         fast_load(*o, fq);
                         fast_poly(fq, rho, P);
                         w = fast_begin(fc, P, dx * ri, dy * ri, (v - start) * iw, o->guess);
