@@ -41,9 +41,10 @@ constexpr int kFastGroup = 64;     // threads that build one row
 struct __align__(16) FastRow {
     float q[kFastD][kFastM]; // coefficient of rho^d cos^m E in P
     float a0[kFastD];        // mean weight over the headings, times the speed's factor exp(-beta w1 v dt (m - m_0))
-    float kappa, rho_max, tol, s; // rho_max = -1: the row is not usable
+    float kappa, tol, tol2, s; // tolerance tol + tol2 rho^2
     float2 guess[kFastGuess];     // F^-1 at 2 pi j / kFastGuess, and the step to the next
-    float pad[4]; // an odd number of 16-byte words: rows of different lanes lie in different banks
+    float rho_max;                // largest rho of the fit; -1: the row is not usable
+    float pad[3]; // an odd number of 16-byte words: rows of different lanes lie in different banks
 };
 
 struct FastPrep {
@@ -129,12 +130,12 @@ struct FastWork {
     float g[kFastGuess / 2 + 1];      // F^-1 on [0, pi]
 };
 
-// The largest rho that a row is fitted on: the error of the cubic fit stays
-// below 2e-6 of the CDF over the whole range of kappa (measured against 64-bit
-// running sums), and below 3e-7 for kappa <= 0.5.
+// The largest rho that a row is fitted on: there the eight harmonics and the
+// cubic fit are off by 2e-6 of the CDF for kappa <= 1, 7e-6 at 2 and 3e-5 at 3
+// (K = 16, against 64-bit running sums), by less and less towards rho = 0.
 __host__ __device__ __forceinline__ float fast_rho_max(float kappa)
 {
-    return fminf(0.3f, 0.2f * fast_rsqrt(fmaxf(fabsf(kappa), 0.1f)));
+    return fminf(0.35f, 0.3f * fast_rsqrt(fmaxf(fabsf(kappa), 0.1f)));
 }
 
 // Builds row `row` of `a` with `nthr` threads (tid < nthr); every thread of
@@ -203,10 +204,11 @@ __host__ __device__ __forceinline__ void fast_row_build(const FastPrep &a, int r
             if (m == kFastM) {
                 o.kappa = kap;
                 o.rho_max = ok ? rmax : -1.0f;
-                // eight harmonics and the cubic fit, the FP32 arithmetic of
-                // both draws, the 2^-22 of ex2.approx and the 2^-24 weights
+                // the FP32 arithmetic of both draws, the 2^-22 of ex2.approx and
+                // the 2^-24 weights, and twice the fit's own error
                 const float k3 = fabsf(kap) * (1.0f / 3.0f), k4 = k3 * k3 * k3 * k3;
-                o.tol = 3.0e-6f + 3.0e-5f * k4 * k4 / fmaxf(k3, 1e-3f);
+                o.tol = 3.0e-6f + 8.0e-6f * k4 * k3 * k3;
+                o.tol2 = (4.0e-6f + 6.0e-5f * k4 * sqrtf(k3)) / (rmax * rmax);
                 o.s = s;
             }
         }

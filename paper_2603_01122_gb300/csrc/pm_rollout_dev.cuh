@@ -1151,7 +1151,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
     // closed-form draw: the lane's row, the squared goal distance it needs and
     // the part of the tolerance that grows with that distance
     const FastRow *row = nullptr;
-    float fkap = 0.0f, ftol = 0.0f, ftol_r = 0.0f, fr2 = INFINITY;
+    float fkap = 0.0f, ftol = 0.0f, ftol2 = 0.0f, ftol_r = 0.0f, fr2 = INFINITY;
     bool wfast = false;
     if (act) {
         const U64x4 r = philox4x64_10(U64x4{i, 0ull, kPurposeSelect, 0ull}, c.seed, c.human);
@@ -1188,6 +1188,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                     ftol_r = fabsf(row->kappa) / row->s;
                     fkap = row->kappa;
                     ftol = row->tol * (float)fc.K;
+                    ftol2 = row->tol2 * (float)fc.K;
                 }
                 fr2 = rmin * rmin * 1.00001f;
                 // the weight-by-weight draw's exponents carry the rounding of
@@ -1301,7 +1302,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                     F2 P[kFastP];
                     FastDraw w;
                     const FastRow *o = row;
-                    float rho, kap = fkap, tol = ftol + far;
+                    float rho, kap = fkap, tol;
                     int base = 0;
                     if constexpr (MS) {
                         float wq[PM_MAX_SPEEDS], total = 0.0f;
@@ -1331,12 +1332,13 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                         base = sp * K;
                         rho = o->s * ri;
                         kap = o->kappa;
-                        tol = fmaf(2.0f * (float)fc.K, o->tol, far) * (total * iw); // (the mean weights carry the same error)
+                        tol = fmaf(1.5f * (float)fc.K, fmaf(o->tol2, rho * rho, o->tol), far) * (total * iw); // (the mean weights carry the same error)
                         fast_load(*o, fq);
                         fast_poly(fq, rho, P);
                         w = fast_begin(fc, P, dx * ri, dy * ri, (v - start) * iw, o->guess);
                     } else {
                         rho = tab.s * ri;
+                        tol = fmaf(ftol2, rho * rho, ftol + far);
                         fast_poly(fq, rho, P);
                         w = fast_begin(fc, P, dx * ri, dy * ri, u, o->guess);
                     }
