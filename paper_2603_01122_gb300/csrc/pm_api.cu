@@ -295,7 +295,7 @@ pm::FastPrep fast_prep(const pm_model *m, const pm::RolloutArgs &a, pm::FastRow 
     f.w1 = m->w1;
     f.w2 = m->w2;
     for (int q = 0; q < f.S; ++q) f.sl[q] = a.tab.S > 0 ? a.tab.sl[q] : a.tab.s;
-    f.rows = pm::fast_applies(m->K, a.enabled, a.tab.S) ? rows : nullptr;
+    f.rows = pm::fast_applies(m->K, a.enabled, __builtin_popcount(a.tab.speed_on)) ? rows : nullptr;
     return f;
 }
 
@@ -449,7 +449,9 @@ pm_status predict_impl(pm_ctx *ctx, const pm_model *model, const float *log_beli
     const size_t words = hist ? (size_t)grid->W * (size_t)grid->H * (size_t)horizon : 0;
     // (the rollout leaves its chunk counter at zero; without `zero` the
     // caller has zeroed the outputs)
-    const pm::FastPrep fp = fast_prep(model, a, model->B <= pm::kFastMaxB ? fast_rows(ctx) : nullptr);
+    // a few steps do not repay the rows (2.5 us where the zeroing does not hide them)
+    const bool rows = model->B <= pm::kFastMaxB && horizon >= 8;
+    const pm::FastPrep fp = fast_prep(model, a, rows ? fast_rows(ctx) : nullptr);
     a.fast = fp.rows;
     const bool z = zero && hist;
     cudaError_t ez = pm::launch_zero_outputs(z ? counts : nullptr, words, z ? oob : nullptr, horizon,

@@ -443,14 +443,14 @@ __global__ void __launch_bounds__(kRowThreads) zero_outputs_kernel(uint32_t *cou
                                                                    unsigned *head, int zblocks,
                                                                    const __grid_constant__ FastPrep fp)
 {
+    // Nothing before the wait: the buffers may have been the inputs of whatever
+    // ran before, and the beta grid its output. The rows are built beside the
+    // zeroing (4.5 us, hidden where 24 MB are zeroed).
+    pdl_wait();
     if ((int)blockIdx.x >= zblocks) {
-        // beside the belief update before this launch: the rows are this
-        // context's, and the beta grid is complete since the update started
         build_rows(fp, ((int)blockIdx.x - zblocks) * kRowsPerCta);
-        pdl_wait(); // the rollout takes this grid's end for the update's end too
         return;
     }
-    pdl_wait(); // the caller's buffers may have been the update's inputs
     const size_t stride = (size_t)zblocks * blockDim.x;
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (counts) {

@@ -353,7 +353,7 @@ __device__ __forceinline__ void posterior_chunk(const PosteriorArgs &a, const Po
 template <bool MS, bool GROUPS>
 __global__ void __launch_bounds__(1024) posterior_kernel(const __grid_constant__ PosteriorArgs a)
 {
-    pdl_release(); // what prepares the rollout may start beside this grid
+    pdl_release(); // what prepares the rollout may be launched beside this grid; it waits for its end
     PostHuman h;
     h.goals = a.goals;
     h.beta = a.beta;

@@ -1141,9 +1141,9 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                                              uint32_t speed_on = 0u)
 {
     const int lane = threadIdx.x & 31;
-    const uint64_t i = (uint64_t)c.i;
-    const bool act = c.i < c.N;
-    const bool trc = c.i < c.n_trace;
+    const uint32_t i = (uint32_t)c.i; // N < 2^31: one register
+    const bool act = i < (uint32_t)c.N;
+    const bool trc = i < (uint32_t)c.n_trace;
     float x = c.z0x, y = c.z0y, cb = 0.0f, gx = 0.0f, gy = 0.0f, cw = 0.0f, bt = 0.0f;
     bool lb = false;
     // several speeds with exactly one enabled: its index (else -1)
@@ -1201,7 +1201,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
         wfast = __all_sync(0xffffffffu, !act || fr2 < INFINITY);
         if (!act) row = c.fast; // an idle lane computes along (any row will do)
     }
-    const size_t plane = (size_t)c.W * (size_t)c.H;
+    const uint32_t plane = (uint32_t)c.W * (uint32_t)c.H; // <= 2^31
     uint32_t *crow = c.counts; // step t's plane of the histogram
     const int xbase = 0x4B400000 + c.cx_off, ybase = 0x4B400000 + c.cy_off;
     // the 32 random bits of step t: a Philox block serves eight steps; beside
@@ -1275,7 +1275,8 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
         if (c.flags) pfkey = (cy >> kFlagShift) * c.fbx + (cx >> kFlagShift);
         ppeers = __match_any_sync(0xffffffffu, pkey);
     };
-    int t = 1, done = 0; // done: steps whose adds are made
+    int t = 1;
+    bool pending = false; // step t-1's adds are still to be made
     while (t <= c.T) {
         uint32_t word = 0u;
         bool open = act;  // step t's draw is still to be made
@@ -1342,10 +1343,8 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                         fast_poly(fq, rho, P);
                         w = fast_begin(fc, P, dx * ri, dy * ri, u, o->guess);
                     }
-                    if (done < t - 1) {
-                        flush(t - 1);
-                        done = t - 1;
-                    }
+                    if (pending) flush(t - 1);
+                    pending = false;
                     k = fast_step(fc, P, rho, kap, tol, w);
                     open = act && (k < 0 || !(r2 > fr2));
                     if (__any_sync(0xffffffffu, open)) {
@@ -1361,6 +1360,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                         k += base;
                     }
                     advance(t, act ? k : 0);
+                    pending = true;
                 }
                 if (t > c.T) break;
                 if (near) open = act; // every lane: the two forms in one step would cost both
@@ -1412,10 +1412,10 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
             }
             advance(t, act ? k : 0);
             flush(t); // at once: its registers are wanted by the next draw
-            done = t++;
+            ++t;
         } while (t <= c.T && (!FAST || !wfast || (near && ((t - 1) & 7) != 0)));
     }
-    if (done < c.T) flush(c.T);
+    if (pending) flush(c.T);
 }
 
 } // namespace pm
