@@ -167,6 +167,7 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
     float4 *comp = reinterpret_cast<float4 *>(slab);
     uint32_t *cdf = reinterpret_cast<uint32_t *>(slab + (size_t)kMaxJ * 16);
     float *betas = reinterpret_cast<float *>(slab + (size_t)kMaxJ * 20); // MS only
+    pdl_wait(); // the zeroed outputs, the rows and the belief
     const int n_items = *a.n_items;
     int cur = -1;
     for (;;) {
@@ -234,6 +235,7 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
             rollout_lane<KT, false, true, true, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words, betas, a.K, h->speed_on);
         else rollout_lane<KT, FULL, false, FAST, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words);
     }
+    release_counter(a.head, lane);
 }
 
 // Two register budgets of the same body: 80 registers (6 CTAs of 128 threads
@@ -315,6 +317,7 @@ __global__ void batch_zero_kernel(const BatchHuman *humans, const int *n_dev)
             for (size_t q = t0; q < nf; q += stride) h.flags[q] = 0u;
         }
     }
+    pdl_release();
 }
 
 // The reachable-cells form. A warp per (human, step t, part g of
@@ -422,6 +425,7 @@ __device__ __forceinline__ void build_rows(const FastPrep &fp, int row0)
 __global__ void __launch_bounds__(kRowThreads) batch_fast_rows_kernel(const BatchHuman *humans, const int *n_dev,
                                                                       const __grid_constant__ FastPrep fp)
 {
+    pdl_wait();
     const int n = *n_dev;
     for (int hh = blockIdx.y; hh < n; hh += gridDim.y) {
         const BatchHuman &h = humans[hh];
@@ -432,6 +436,7 @@ __global__ void __launch_bounds__(kRowThreads) batch_fast_rows_kernel(const Batc
         const int row0 = blockIdx.x * kRowsPerCta;
         if (h.B <= kFastMaxB && row0 < h.B * fp.S) build_rows(p, row0); // the same for the whole CTA
     }
+    pdl_release();
 }
 
 // The single-human form of the above: the counts in 16-byte words (scalar
@@ -481,6 +486,7 @@ cudaError_t launch_or_query(Kern k, const BatchArgs &a, int blocks, int threads,
     }
     if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, threads, dyn);
     cudaGetLastError();
+    if (a.early) return launch_early(k, (unsigned)blocks, (unsigned)threads, dyn, s, a);
     k<<<blocks, threads, dyn, s>>>(a);
     return cudaGetLastError();
 }
@@ -586,10 +592,12 @@ cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, i
 }
 
 cudaError_t launch_batch_fast_rows(const BatchHuman *humans, const int *n_dev, int max_rows, const FastPrep &fp,
-                                   cudaStream_t s)
+                                   bool early, cudaStream_t s)
 {
     if (max_rows <= 0) return cudaSuccess;
     const dim3 grid((kFastMaxB * fp.S + kRowsPerCta - 1) / kRowsPerCta, (unsigned)std::min(max_rows, 1024));
+    cudaGetLastError();
+    if (early) return launch_early(batch_fast_rows_kernel, grid, kRowThreads, 0, s, humans, n_dev, fp);
     batch_fast_rows_kernel<<<grid, kRowThreads, 0, s>>>(humans, n_dev, fp);
     return cudaGetLastError();
 }
@@ -606,7 +614,11 @@ cudaError_t launch_batch_zero(const BatchHuman *humans, const int *n_dev, int ma
         batch_zero_reach_kernel<<<(unsigned)std::max<long>(ctas, 1), 256, 0, s>>>(humans, n_dev, prev, ticket, smax);
         return cudaGetLastError();
     }
-    dim3 grid((unsigned)(sm_count * 2), (unsigned)(max_rows < 64 ? max_rows : 64));
+    // 16 CTAs an SM in all, some stores a thread: with sm_count * 2 CTAs for
+    // each of 64 humans of 0.8 MB (19,456 CTAs) their launch was what took the
+    // time (20 -> 9.5 us)
+    const int rows = max_rows < 64 ? max_rows : 64;
+    const dim3 grid((unsigned)std::max(std::min(sm_count * 2, sm_count * 16 / rows), 1), (unsigned)rows);
     batch_zero_kernel<<<grid, 256, 0, s>>>(humans, n_dev);
     return cudaGetLastError();
 }

@@ -143,14 +143,14 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... Params, typename... Args>
-cudaError_t launch_early(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t dyn, cudaStream_t s,
+cudaError_t launch_early(void (*kernel)(Params...), dim3 blocks, unsigned threads, size_t dyn, cudaStream_t s,
                          Args... args)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = blocks;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = dyn;
     cfg.stream = s;

@@ -177,7 +177,8 @@ struct BatchArgs {
     const BatchHuman *humans;
     const int2 *items;   // (human, first particle), longest horizon first
     const int *n_items;
-    unsigned *head;      // next tile (zeroed before every launch)
+    unsigned *head;      // next tile (the warp form leaves it at zero, the window form does not)
+    int early;           // launched right after the zeroing, on its stream: may overlap its end
     int win_radius_cap;  // (2r+1)^2 cells fit the dynamic shared memory
     unsigned *status;    // context status word (or NULL)
     int marks;           // write block occupancy flags (the humans' flags are set)
@@ -228,7 +229,7 @@ cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, i
 // The rows of every human of a batch with at most kFastMaxB beta values
 // (fp: B and beta per human).
 cudaError_t launch_batch_fast_rows(const BatchHuman *humans, const int *n_dev, int max_rows, const FastPrep &fp,
-                                   cudaStream_t s);
+                                   bool early, cudaStream_t s);
 size_t adjoint_scratch_bytes(int M, int G, int J);
 void adjoint_scratch_layout(void *base, int M, int G, int J, AdjointArgs &a);
 

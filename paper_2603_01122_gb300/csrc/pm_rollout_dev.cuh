@@ -924,6 +924,20 @@ __device__ __forceinline__ int draw_multi_lb(const HeadingTab &tab, uint32_t spe
     return qs * KT + kk;
 }
 
+// Every warp leaves the chunk loop once, after its last (failed) grab; the
+// last one to leave resets the counter head[0] and its own count head[2], so
+// each launch finds both at zero without a memset before it (the counters
+// are zeroed when the context or the batch allocates them).
+__device__ __forceinline__ void release_counter(unsigned *head, int lane)
+{
+    if (lane != 0) return;
+    const unsigned warps = gridDim.x * (blockDim.x >> 5);
+    if (atomicAdd(head + 2, 1u) == warps - 1u) {
+        atomicExch(head, 0u);
+        atomicExch(head + 2, 0u);
+    }
+}
+
 // Per-tile state of one human for rollout_tile.
 struct TileCtx {
     float z0x, z0y;
