@@ -828,10 +828,10 @@ pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream, bool after_zero =
     a.status = status_word(ctx);
     a.marks = (b->block_flags && b->warp_hist && b->d_flags) ? 1 : 0;
     a.fc = t.fc;
-    if (b->d_fast && b->warp_hist) {
-        a.fast = b->d_fast;
-        e = pm::launch_batch_fast_rows(b->d_humans, b->d_meta + 1, b->max_humans, fast_prep(&b->shared, t, b->d_fast),
-                                       after_zero, stream);
+    const pm::FastPrep fp = fast_prep(&b->shared, t, b->warp_hist ? b->d_fast : nullptr);
+    if (fp.rows) {
+        a.fast = fp.rows;
+        e = pm::launch_batch_fast_rows(b->d_humans, b->d_meta + 1, b->max_humans, fp, after_zero, stream);
         if (e != cudaSuccess) return cuda_fail(e, "rows of the closed-form draw");
     }
     const size_t dyn = batch_dyn_smem(b);
@@ -842,7 +842,7 @@ pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream, bool after_zero =
     if (b->ctas_per_sm > 0) occ = std::min(occ, b->ctas_per_sm);
     // (behind the rows kernel the early launch placed the persistent CTAs around
     // its last ones: 16 humans 3.07 ms against 2.99)
-    a.early = after_zero && b->warp_hist && !b->d_fast ? 1 : 0;
+    a.early = after_zero && b->warp_hist && !fp.rows ? 1 : 0;
     e = pm::launch_batch_rollout(a, batch_shape_of(b), ctx->sm_count * occ, dyn, stream);
     if (e != cudaSuccess) return cuda_fail(e, "batch rollout launch");
     // (the warp form's last warp has left the tile counter at zero)

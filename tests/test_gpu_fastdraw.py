@@ -65,9 +65,10 @@ def test_equals_weight_by_weight(K, speeds, off, dt, b_lo, b_hi, near, traced):
         assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("K,speeds", [(36, None), (20, None), (64, None), (32, (0.5, 1.0, 1.5))])
+@pytest.mark.parametrize("K,speeds,off", [(36, None, 0), (20, None, 0), (64, None, 0), (32, (0.5, 1.0, 1.5), 0),
+                                          (16, (0.5, 1.0, 1.5), 0b110)])  # the last: too few controls left for rows
 @pytest.mark.parametrize("marks", [0, 1])
-def test_batch_equals_weight_by_weight(K, speeds, marks):
+def test_batch_equals_weight_by_weight(K, speeds, off, marks):
     rng = np.random.default_rng(K + 1)
     n, B, T, W, H = 5, 9, 40, 61, 67
     outs = []
@@ -78,7 +79,7 @@ def test_batch_equals_weight_by_weight(K, speeds, marks):
         ctx = pm.pm_create(0)
         try:
             b = torch.tensor(np.append(beta, np.ones(pad, np.float32))).cuda()
-            model = pm.make_model(K, 1.0, 0.03, goals[0], b, speeds=speeds)
+            model = pm.make_model(K, 1.0, 0.03, goals[0], b, speeds=speeds, speed_off=off)
             batch = pm.pm_batch_create(ctx, model, n)
             z0 = torch.zeros((n, 2), device="cuda")
             lb = [torch.tensor(np.pad(p, ((0, 0), (0, pad)), constant_values=-np.inf).ravel()).cuda() for p in belief]
