@@ -36,6 +36,9 @@ sys.path.insert(0, ROOT)
 
 import workloads  # noqa: E402
 
+# Warp instructions per warp-step of the rollout with the closed-form draw (ncu, smsp__inst_executed)
+ISSUE_PER_WARP_STEP = {"one speed": 244, "several speeds": 348}
+ISSUE_PEAK = 4 * 152 * 2.07e9  # one warp instruction per clock and scheduler
 METRIC = "particle-steps/s"
 
 
@@ -54,7 +57,8 @@ HBM_PEAK_GBS = _measured_peak("hbm_gbs", 6794.5)
 # reaches them only through pm_limits.h; the traffic of a
 # committed ncu summary is used only while these are unchanged)
 ROLLOUT_SOURCES = ["paper_2603_01122_gb300/csrc/pm_rollout.cu", "paper_2603_01122_gb300/csrc/pm_rollout_dev.cuh",
-                   "paper_2603_01122_gb300/csrc/pm_internal.cuh", "include/pm_limits.h"]
+                   "paper_2603_01122_gb300/csrc/pm_internal.cuh", "include/pm_limits.h",
+                   "paper_2603_01122_gb300/csrc/pm_fastdraw.cuh"]
 
 
 # main-line workloads: generator and the rollout kernel that dominates it
@@ -482,7 +486,7 @@ def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
                           "speedup_vs_plain": plain_ms / batch_ms, "autotune_s": tune_s,
                           "tuned": tuned,
                           "rate_vs_plain_small": steps / (batch_ms * 1e-3) / out["plain_small"]["particle_steps_per_s"],
-                          "sfu_roofline_frac": steps / (batch_ms * 1e-3) * 2 * 36 / sfu_peak,
+                          "issue_roofline_frac": steps / (batch_ms * 1e-3) / 32 * ISSUE_PER_WARP_STEP["one speed"] / ISSUE_PEAK,
                           "union": {"ms": union_ms, "sigma_cells": 1.5, "bytes": union_bytes,
                                     "GB_per_s": union_bytes / (union_ms * 1e-3) / 1e9,
                                     "hbm_frac": union_bytes / (union_ms * 1e-3) / 1e9 / HBM_PEAK_GBS,
@@ -600,7 +604,7 @@ def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
                 "particle_steps_per_frame": ps, "particle_steps_per_s": ps / float(np.median(lat)),
                 "plain_path_ms_per_frame": plain_ms, "speedup_vs_plain": plain_ms / float(np.median(lat) * 1e3),
                 "rate_vs_plain_small": ps / float(np.median(lat)) / out["plain_small"]["particle_steps_per_s"],
-                "sfu_roofline_frac": ps / float(np.median(lat)) * 2 * 36 / sfu_peak}
+                "issue_roofline_frac": ps / float(np.median(lat)) / 32 * ISSUE_PER_WARP_STEP["one speed"] / ISSUE_PEAK}
             # the same frames with the grid epilogue (blur + max-union on the room grid) in the graph
             srv_u = Server(ctx, hu0.K, hu0.speed, hu0.dt, hu0.grid, max_live=64, n_particles=hu0.n_particles,
                            horizon=hu0.horizon, window=hu0.window, union_sigma=1.5)
@@ -685,7 +689,7 @@ def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
             u_on = hu.K * sum(1 for q in range(len(hu.speeds)) if not (hu.speed_off >> q) & 1)
             rate = hu.n_particles * hu.horizon / (ms * 1e-3)
             out[name] = {"ms_per_prediction": ms, "particle_steps_per_s": rate, "controls_enabled": u_on,
-                         "sfu_roofline_frac": rate * 2 * u_on / sfu_peak}
+                         "issue_roofline_frac": rate / 32 * ISSUE_PER_WARP_STEP["several speeds"] / ISSUE_PEAK}
 
     if want("table1"):
         # -- Table 1's configuration (1 human, n = 8192, |G| = 10, |B| = 5, |U| = 96,
@@ -751,18 +755,18 @@ def sig(x, n=4):
 
 
 def target_summary(line, extra):
-    """The figures the targets are stated in, compact: the rollout's SFU
-    fraction, the batched and served rates against the plain per-human path
+    """The figures the targets are stated in, compact: the rollout's
+    roofline fraction, the batched and served rates against the plain per-human path
     (the plain configuration's rate, and the same humans issued one by one,
     also for 64 humans of the plain configuration's shape) and the 64-human
     frame latency with and without the grid epilogue."""
-    t = {"rollout_sfu_frac": sig(line["roofline"]["frac"], 3), "value": sig(line["value"])}
+    t = {"rollout_frac": sig(line["roofline"]["frac"], 3), "value": sig(line["value"])}
     if not extra:
         return t
     t["plain_small_rate"] = sig(extra["plain_small"]["particle_steps_per_s"])
     b = extra.get("batched")
     if b:
-        t["batched"] = {"rate": sig(b["batched_particle_steps_per_s"]), "sfu_frac": sig(b["sfu_roofline_frac"], 3),
+        t["batched"] = {"rate": sig(b["batched_particle_steps_per_s"]), "issue_frac": sig(b["issue_roofline_frac"], 3),
                         "x_plain_small": sig(b["rate_vs_plain_small"], 3),
                         "x_same_humans_one_by_one": sig(b["speedup_vs_plain"], 3), "ms": sig(b["batched_ms"])}
     c = extra.get("batched_small")
@@ -774,7 +778,7 @@ def target_summary(line, extra):
         t["served_64"] = {"p50_ms": sig(f["p50_ms"]), "p99_ms": sig(f["p99_ms"]),
                           "with_union_p99_ms": sig(f.get("with_union", {}).get("p99_ms")),
                           "with_union_p50_ms": sig(f.get("with_union", {}).get("p50_ms")),
-                          "rate": sig(f["particle_steps_per_s"]), "sfu_frac": sig(f["sfu_roofline_frac"], 3),
+                          "rate": sig(f["particle_steps_per_s"]), "issue_frac": sig(f["issue_roofline_frac"], 3),
                           "x_plain_small": sig(f["rate_vs_plain_small"], 3),
                           "x_same_humans_one_by_one": sig(f["speedup_vs_plain"], 3)}
     p = extra.get("serving_poisson")
@@ -785,7 +789,7 @@ def target_summary(line, extra):
         t["adjoint_ms"] = sig(d["ms_per_backward"])
     m = extra.get("multi_speed")
     if m:
-        t["multi_speed_sfu_frac"] = sig(m["sfu_roofline_frac"], 3)
+        t["multi_speed_issue_frac"] = sig(m["issue_roofline_frac"], 3)
     return t
 
 
@@ -907,9 +911,23 @@ def run_native(args):
     # per launch (one exp + one sqrt per control and particle-step) / its
     # event-timed duration
     roll_avg_s = statistics.mean(roll_ms) * 1e-3
-    sfu_ops = 2.0 * U * N * T
-    achieved = sfu_ops / roll_avg_s / 1e9
-    peak = 2.0 / (1.0 / sfu["ex2"] + 1.0 / sfu["sqrt"]) / 1e9
+    # (the closed-form draw, K >= 20 headings or several speeds, forms neither:
+    # its rollout is bound by instruction issue, counted by ncu)
+    closed = hu.K >= 16 and U >= 20 and len(hu.beta) <= 16 and not getattr(hu, "heading_off", 0)
+    if closed:
+        instr = ISSUE_PER_WARP_STEP["several speeds" if U > hu.K else "one speed"]
+        achieved = instr * ((N + 31) // 32) * T / roll_avg_s / 1e9
+        peak = ISSUE_PEAK / 1e9
+        unit, source = "G warp instructions/s", "one per clock and scheduler, 152 SMs x 4 at 2070 MHz"
+        algorithmic = f"{instr} warp instructions per warp-step (ncu, profiles/rollout_paper_scale.md)"
+    else:
+        sfu_ops = 2.0 * U * N * T
+        achieved = sfu_ops / roll_avg_s / 1e9
+        peak = 2.0 / (1.0 / sfu["ex2"] + 1.0 / sfu["sqrt"]) / 1e9
+        unit = "G SFU results/s"
+        source = ("measured by pm_probe_sfu (ex2/sqrt 1:1 harmonic mean); "
+                  f"ex2 {sfu['ex2'] / 1e9:.1f}, sqrt {sfu['sqrt'] / 1e9:.1f}, rsqrt {sfu['rsqrt'] / 1e9:.1f} G/s")
+        algorithmic = f"2U SFU results (U = {U} controls: U ex2 + U sqrt) per particle-step"
     khash = sources_hash(ROLLOUT_SOURCES)
     traffic = load_profile_traffic(khash, args.workload)
 
@@ -966,17 +984,13 @@ def run_native(args):
             "scaling": "weak", "vs_baseline": None, "dtype": "f32",
             "data": "synthetic (seeded; observed history drawn from the model on the GPU)",
             "config": workload_config(hu, args.workload),
-            # per step: the belief update, the zeroing of the outputs, the rollout
-            "gpu_launches": 3 * args.steps,
+            # per step: the belief update, the zeroing of the outputs, the rows of the closed-form draw, the rollout
+            "gpu_launches": (4 if closed else 3) * args.steps,
             "wall_s": wall,
             "breakdown_ms": {"posterior": statistics.mean(post_ms), "rollout": statistics.mean(roll_ms)},
             "roofline": {"bound": "alu", "kernel": kernel_name, "achieved": achieved,
-                         "peak": peak, "unit": "G SFU results/s", "frac": achieved / peak,
-                         "traffic": traffic,
-                         "peak_source": "measured by pm_probe_sfu (ex2/sqrt 1:1 harmonic mean); "
-                                        f"ex2 {sfu['ex2'] / 1e9:.1f}, sqrt {sfu['sqrt'] / 1e9:.1f}, "
-                                        f"rsqrt {sfu['rsqrt'] / 1e9:.1f} G/s",
-                         "algorithmic": f"2U SFU results (U = {U} controls: U ex2 + U sqrt) per particle-step"},
+                         "peak": peak, "unit": unit, "frac": achieved / peak, "traffic": traffic,
+                         "peak_source": source, "algorithmic": algorithmic},
             "device": info,
             "clocks": {**clk.summary(), "window": f"{pre} pre-roll steps + the timed region"},
             "e2e": {"value": e2e_value, "unit": METRIC, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
@@ -987,7 +1001,7 @@ def run_native(args):
         }
         extra = None
         if not args.no_extra:
-            extra = run_extra(args, pm, ctx, torch, dev, stream, peak * 1e9)
+            extra = run_extra(args, pm, ctx, torch, dev, stream, 2.0 / (1.0 / sfu["ex2"] + 1.0 / sfu["sqrt"]))
             line["extra"] = extra
         if not args.no_cpu_baseline:
             threads = host_threads()

@@ -249,7 +249,9 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 3) batch_warp_kernel(const _
 }
 
 // With the closed-form draw. One speed, K <= 36: 80 registers (6 CTAs of 128
-// threads per SM); K = 64 and several speeds: 96 (5 CTAs), fewer spills.
+// threads per SM; 96 registers and 5 CTAs: a frame of 64 humans 5.17 ms against
+// 4.91); K = 64 and several speeds: 96, for fewer spills (31 humans of 96
+// controls 2.06 ms against 2.26).
 template <int KT, bool FULL, bool MS, bool MARKS>
 __global__ void __maxnreg__((MS || KT == 64) ? 96 : 80) batch_fast_kernel(const __grid_constant__ BatchArgs a)
 {
