@@ -37,7 +37,7 @@ sys.path.insert(0, ROOT)
 import workloads  # noqa: E402
 
 # Warp instructions per warp-step of the rollout with the closed-form draw (ncu, smsp__inst_executed)
-ISSUE_PER_WARP_STEP = {"one speed": 244, "several speeds": 348}
+ISSUE_PER_WARP_STEP = {"one speed": 239, "several speeds": 343}
 ISSUE_PEAK = 4 * 152 * 2.07e9  # one warp instruction per clock and scheduler
 METRIC = "particle-steps/s"
 
