@@ -19,9 +19,11 @@
 //
 // The result is used only where x lies clear of a whole number by more than
 // the error of this evaluation and of the weight-by-weight draw together
-// (`tol` below); the lanes that are closer (one in some 10^4 at K = 36) take
-// the weight-by-weight draw, so the chosen heading is always the one that the
-// fixed-point weights give.
+// (`tol` below); the lanes that are closer (at least 2 K tol of them: one in
+// 4600 or more at K = 36) take the weight-by-weight draw, so the chosen
+// heading is always the one that the fixed-point weights give. A goal so far
+// away that those weights lose bits keeps the weight-by-weight draw
+// (rollout_lane).
 #pragma once
 
 #include "pm_internal.cuh"

@@ -1190,14 +1190,17 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
             if (c.fast) {
                 row = c.fast + (size_t)(lo % c.B) * (MS ? tab.S : 1);
                 float rmin = 0.0f; // the goal distance below which a row no longer holds
+                float smax = 0.0f; // the longest step
                 if constexpr (MS) {
                     for (int q = 0; q < tab.S; ++q)
                         if ((speed_on >> q) & 1u) {
                             const float rm = row[q].rho_max;
                             rmin = fmaxf(rmin, rm > 0.0f ? row[q].s / rm : INFINITY);
                             ftol_r = fmaxf(ftol_r, fabsf(row[q].kappa) / row[q].s);
+                            smax = fmaxf(smax, row[q].s);
                         }
                 } else {
+                    smax = row->s;
                     rmin = row->rho_max > 0.0f ? row->s / row->rho_max : INFINITY;
                     ftol_r = fabsf(row->kappa) / row->s;
                     fkap = row->kappa;
@@ -1205,9 +1208,18 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                     ftol2 = row->tol2 * (float)fc.K;
                 }
                 fr2 = rmin * rmin * 1.00001f;
-                // the weight-by-weight draw's exponents carry the rounding of
-                // beta w2 r: some 2^-24 of it after its residual correction
+                // the weight-by-weight draw's exponents carry a rounding of
+                // beta w2 r: the 2^-23 of the approximate square root times
+                // the 1.8e-3 of its correction's factor, and twice that
                 ftol_r *= 4e-10f * (float)fc.K;
+                // Its reference distance lies 2^-20 r beyond the bound
+                // (lb_step_d), so the largest of its 23-bit weights is
+                // 2^(-|cb| 2^-20 r) smaller. Up to half a bit is within the
+                // tolerance; where a particle may get farther the closed
+                // form would be the more exact one, but not the same one.
+                const float dx = x - gx, dy = y - gy;
+                const float far = sqrt_approx(fmaf(dx, dx, dy * dy)) + (float)c.T * smax;
+                if (!(fabsf(cb) * far <= 0x1p19f)) fr2 = INFINITY;
             }
         }
     }

@@ -97,3 +97,22 @@ def test_batch_equals_weight_by_weight(K, speeds, off, marks):
         finally:
             pm.pm_destroy(ctx)
     assert np.array_equal(outs[0][0], outs[1][0]) and np.array_equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("K,speeds", [(20, None), (36, None), (64, None), (32, (0.5, 1.0, 1.5))])
+@pytest.mark.parametrize("away", [1e3, 1e4, 3e5, 1e7])
+def test_far_goals_equal_weight_by_weight(K, speeds, away):
+    """Goals so far away that the rounding of beta |z - g| shows in the fixed-point weights."""
+    rng = np.random.default_rng(K)
+    G, B, N, T, W, H, res, z0 = 2, 16, 6001, 33, 61, 61, 0.1, (1.5, -0.5)
+    goals = (np.array(z0) + away * np.array([[0.6, 0.8], [-1.0, 0.3]])).astype(np.float32)
+    beta = (10.0 ** np.linspace(-2.0, 1.5, B)).astype(np.float32)
+    beta[::3] *= -1.0
+    log_b = np.log(rng.dirichlet(np.ones(G * B))).astype(np.float32)
+    wide = np.full((G, B + 1), -np.inf, np.float32)
+    wide[:, :B] = log_b.reshape(G, B)
+    args = (0.05, N, T, W, H, res, z0, True)
+    got = _predict(K, speeds, 0, goals, beta, log_b, *args)
+    want = _predict(K, speeds, 0, goals, np.append(beta, np.float32(1.0)), wide.ravel(), *args)
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
