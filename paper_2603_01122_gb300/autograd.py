@@ -37,15 +37,18 @@ class MarginalLogLik(torch.autograd.Function):
         if any(fctx.needs_input_grad[:3]):
             grad = torch.empty(goals_c.numel() + 3, dtype=torch.float64, device=goals.device)
             pm_loglik_value_grad(*args, grad, stream)
-            # the inputs too: a change to them before backward is refused, as ever
-            fctx.save_for_backward(grad, goals_c, speed, w, beta, offsets, traj, log_prior)
         else:
+            grad = None  # backward may still run, for beta, traj or log_prior: they get no gradient
             pm_loglik_forward(*args, stream)
+        # the inputs too: a change to them before backward is refused, as ever
+        fctx.save_for_backward(grad, goals_c, speed, w, beta, offsets, traj, log_prior)
         return out
 
     @staticmethod
     def backward(fctx, grad_out):
         grad, goals, speed, w = fctx.saved_tensors[:4]
+        if grad is None:
+            return (None,) * 12
         d = (grad * grad_out.detach().to(torch.float64)).to(torch.float32)
         n = goals.numel()
         need = fctx.needs_input_grad

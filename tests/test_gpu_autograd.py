@@ -1,0 +1,66 @@
+"""The autograd function's contract: which inputs may ask for a gradient, what is refused, what a value costs."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2603_01122_gb300 as pm
+from gpu_util import dev
+from paper_2603_01122_gb300 import autograd
+from paper_2603_01122_gb300.autograd import MarginalLogLik, marginal_loglik
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = pm.pm_create(0)
+    yield c
+    pm.pm_destroy(c)
+
+
+def _inputs():
+    """Two short walks, G = 2, B = 3: goals, speed, w, beta, offsets, traj, log_prior."""
+    rng = np.random.default_rng(5)
+    th = rng.uniform(0.0, 6.28, (2, 9))
+    step = 0.1 * np.stack([np.cos(th), np.sin(th)], -1)
+    traj = np.concatenate([np.concatenate([[[1.0, 2.0]], [1.0, 2.0] + np.cumsum(s, 0)]) for s in step])
+    return dict(goals=dev(rng.uniform(0.0, 5.0, (2, 2))), speed=torch.tensor(1.0).cuda(),
+                w=torch.tensor([1.0, 1.0]).cuda(), beta=dev([0.5, 1.0, 4.0]),
+                offsets=dev(np.array([0, 10, 20], np.int32), torch.int32), traj=dev(traj),
+                log_prior=dev(np.full(6, -np.log(6.0))))
+
+
+def _call(ctx, p, f=marginal_loglik):
+    args = (p["goals"], p["speed"], p["w"], p["beta"], 12, 0.1, p["offsets"], p["traj"], p["log_prior"], ctx)
+    return f(*args)
+
+
+@pytest.mark.parametrize("which", [("beta",), ("traj",), ("log_prior",), ("beta", "goals"), ("w",), ("speed", "traj")])
+def test_any_input_may_require_a_gradient(ctx, which):
+    """goals, speed and w get theirs; the data get none, alone or beside them."""
+    p = _inputs()
+    for k in which:
+        p[k].requires_grad_()
+    L = _call(ctx, p)
+    L.backward()
+    full = _inputs()
+    for k in ("goals", "speed", "w"):
+        full[k].requires_grad_()
+    L_full = _call(ctx, full)
+    L_full.backward()
+    assert torch.equal(L, L_full)
+    for k in p:
+        if k in which and k in ("goals", "speed", "w"):
+            assert torch.equal(p[k].grad, full[k].grad)
+        else:
+            assert p[k].grad is None
+
+
+@pytest.mark.parametrize("which", ["goals", "beta"])
+def test_input_changed_before_backward_is_refused(ctx, which):
+    p = _inputs()
+    p[which].requires_grad_()
+    L = _call(ctx, p)
+    p["traj"].add_(1.0)
+    with pytest.raises(RuntimeError, match="modified by an inplace operation"):
+        L.backward()
