@@ -6,7 +6,8 @@ scalar). Where a gradient is wanted, the forward call takes L and the gradient
 with respect to the goal coordinates, the speed and the Q weights from one
 pass of the adjoint kernel (it forms both from the same weights; a second
 pass in backward cost as much again), and backward scales it on the device,
-in FP64 before the rounding to FP32, without a word read back to the host.
+in FP64 before the rounding to FP32. An incoming gradient that is not finite
+is refused (PM_EINVAL), as pm_loglik_backward refuses it.
 ``speed`` and ``w`` are read to the host once per call (the C ABI takes them
 as scalars). ``speeds`` (a tuple of multipliers, or None for one speed)
 selects the control set of several speeds; ``snap_heading`` reads each
@@ -15,9 +16,11 @@ B = 10, value and gradient: 450 -> 360 us.
 """
 from __future__ import annotations
 
+import math
+
 import torch
 
-from . import make_model, pm_loglik_forward, pm_loglik_value_grad
+from . import PM_EINVAL, PmError, make_model, pm_loglik_forward, pm_loglik_value_grad
 
 
 class MarginalLogLik(torch.autograd.Function):
@@ -47,15 +50,21 @@ class MarginalLogLik(torch.autograd.Function):
     @staticmethod
     def backward(fctx, grad_out):
         grad, goals, speed, w = fctx.saved_tensors[:4]
-        if grad is None:
-            return (None,) * 12
-        d = (grad * grad_out.detach().to(torch.float64)).to(torch.float32)
-        n = goals.numel()
-        need = fctx.needs_input_grad
-        gg = d[:n].view(goals.shape) if need[0] else None
-        gs = d[n:n + 1].to(speed.device).reshape(speed.shape) if need[1] else None
-        gw = d[n + 1:].to(w.device).reshape(w.shape) if need[2] else None
-        return gg, gs, gw, None, None, None, None, None, None, None, None, None
+        out = [None] * 12
+        if grad is not None:
+            d = (grad * grad_out.detach()).to(torch.float32)  # the product in FP64
+            n = goals.numel()
+            need = fctx.needs_input_grad
+            if need[0]:
+                out[0] = d[:n].view(goals.shape)
+            if need[1]:
+                out[1] = d[n:n + 1].to(speed.device).reshape(speed.shape)
+            if need[2]:
+                out[2] = d[n + 1:].to(w.device).reshape(w.shape)
+        # read back after the work above is queued: what waits for it is the check alone
+        if not math.isfinite(grad_out.item()):
+            raise PmError(PM_EINVAL, "grad_out must be finite")
+        return tuple(out)
 
 
 def marginal_loglik(goals, speed, w, beta, K, dt, offsets, traj, log_prior, ctx, speeds=None, snap_heading=False):

@@ -64,3 +64,14 @@ def test_input_changed_before_backward_is_refused(ctx, which):
     p["traj"].add_(1.0)
     with pytest.raises(RuntimeError, match="modified by an inplace operation"):
         L.backward()
+
+
+@pytest.mark.parametrize("g", [float("inf"), float("nan")])
+@pytest.mark.parametrize("which", ["goals", "beta"])
+def test_non_finite_gradient_is_refused(ctx, which, g):
+    p = _inputs()
+    p[which].requires_grad_()
+    with pytest.raises(pm.PmError, match="grad_out must be finite") as e:
+        (g * _call(ctx, p)).backward()
+    assert e.value.status == pm.PM_EINVAL
+    assert p[which].grad is None
