@@ -2,7 +2,8 @@
 
 ``MarginalLogLik.apply(goals, speed, w, beta, K, dt, offsets, traj, log_prior, ctx, speeds, snap_heading)``
 returns the marginal log-likelihood L of the observed trajectories (a CUDA
-scalar). Where a gradient is wanted, the forward call takes L and the gradient
+scalar). Where a gradient is wanted (an input requires one and the grad mode is
+on), the forward call takes L and the gradient
 with respect to the goal coordinates, the speed and the Q weights from one
 pass of the adjoint kernel (it forms both from the same weights; a second
 pass in backward cost as much again), and backward scales it on the device,
@@ -24,6 +25,14 @@ from . import PM_EINVAL, PmError, make_model, pm_loglik_forward, pm_loglik_value
 
 
 class MarginalLogLik(torch.autograd.Function):
+    @classmethod
+    def apply(cls, *args):
+        # needs_input_grad is about the inputs alone, whatever the grad mode,
+        # and forward always runs with it off: a value-only call is seen here
+        if not torch.is_grad_enabled():
+            args = tuple(a.detach() if isinstance(a, torch.Tensor) else a for a in args)
+        return super().apply(*args)
+
     @staticmethod
     def forward(fctx, goals, speed, w, beta, K, dt, offsets, traj, log_prior, ctx, speeds=None, snap_heading=False):
         v_t, w_t = speed.detach().reshape(1), w.detach().reshape(2)

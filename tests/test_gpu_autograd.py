@@ -75,3 +75,20 @@ def test_non_finite_gradient_is_refused(ctx, which, g):
         (g * _call(ctx, p)).backward()
     assert e.value.status == pm.PM_EINVAL
     assert p[which].grad is None
+
+
+@pytest.mark.parametrize("call", [marginal_loglik, MarginalLogLik.apply])
+@pytest.mark.parametrize("mode", [torch.no_grad, torch.inference_mode])
+def test_value_without_grad_mode_takes_no_gradient_pass(ctx, monkeypatch, call, mode):
+    p = _inputs()
+    for k in ("goals", "speed", "w"):
+        p[k].requires_grad_()
+    want = _call(ctx, p)
+
+    def refuse(*_):
+        raise AssertionError("gradient pass in a value-only call")
+
+    monkeypatch.setattr(autograd, "pm_loglik_value_grad", refuse)
+    with mode():
+        got = _call(ctx, p, call)
+    assert torch.equal(got, want) and not got.requires_grad
