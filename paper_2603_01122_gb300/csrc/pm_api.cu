@@ -358,13 +358,23 @@ pm_status ensure_stage(pm_ctx *ctx, size_t bytes)
 unsigned *status_word(pm_ctx *ctx) { return ctx->ticket ? ctx->ticket + 3 : nullptr; }
 
 // The context's rows of the closed-form draw (kFastMaxB * PM_MAX_SPEEDS).
+constexpr size_t kFastRowBytes = sizeof(pm::FastRow) * pm::kFastMaxB * PM_MAX_SPEEDS;
 pm::FastRow *fast_rows(pm_ctx *ctx) { return reinterpret_cast<pm::FastRow *>(ctx->ticket + 64); }
+
+// A component's folded log-belief per component (kMaxJ), for the belief
+// update's groups: of one size for every call, so that the scratch below grows
+// with the partial sums alone (growing it frees what a captured graph may hold,
+// and is not possible inside a capture).
+float2 *fold_scratch(pm_ctx *ctx)
+{
+    return reinterpret_cast<float2 *>(reinterpret_cast<char *>(fast_rows(ctx)) + kFastRowBytes);
+}
 
 pm_status ensure_posterior_scratch(pm_ctx *ctx, size_t bytes)
 {
     if (!ctx->ticket) {
-        // the counter block, then the rows of the closed-form draw
-        cudaError_t e = cudaMalloc((void **)&ctx->ticket, 256 + sizeof(pm::FastRow) * pm::kFastMaxB * PM_MAX_SPEEDS);
+        // the counter block, the rows of the closed-form draw, the groups' folded components
+        cudaError_t e = cudaMalloc((void **)&ctx->ticket, 256 + kFastRowBytes + pm::kMaxJ * sizeof(float2));
         if (e == cudaSuccess) e = cudaMemset(ctx->ticket, 0, 256);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -489,9 +499,7 @@ pm_status posterior_impl(pm_ctx *ctx, const pm_model *model, const float *obs_xy
     a.log_prior = log_prior;
     a.log_b = log_belief;
     const int n_chunks = pm::posterior_chunks(n_obs, &a.steps_per_chunk);
-    // the partial sums, then (at an 8-byte boundary) the groups' folded components
-    const size_t part = (pm::posterior_scratch_bytes(n_chunks, model->G * model->B) + 7) & ~(size_t)7;
-    st = ensure_posterior_scratch(ctx, part + J * sizeof(float2));
+    st = ensure_posterior_scratch(ctx, pm::posterior_scratch_bytes(n_chunks, model->G * model->B));
     if (st != PM_OK) return st;
     a.part = (float *)ctx->post_scratch;
     a.ticket = ctx->ticket;
@@ -499,7 +507,7 @@ pm_status posterior_impl(pm_ctx *ctx, const pm_model *model, const float *obs_xy
     // a chunk (256 components, 200 steps: 85 us with 32 warps a chunk,
     // 32 us with eight times as many)
     a.groups = (int)((J + 31) / 32);
-    a.fold = (float2 *)((char *)ctx->post_scratch + part);
+    a.fold = fold_scratch(ctx);
     a.gticket = ctx->ticket + 16;
     a.status = status_word(ctx);
     cudaError_t e = pm::launch_posterior(a, n_chunks, stream);

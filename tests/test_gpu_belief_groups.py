@@ -42,3 +42,47 @@ def test_groups_equal_one_cta(G, B, n_obs, moving, speeds):
         pm.pm_batch_destroy(batch)
     finally:
         pm.pm_destroy(ctx)
+
+
+def test_scratch_of_a_long_history_serves_many_components_in_a_capture():
+    """64 chunks of 4 components need as many partial sums as one chunk of 256:
+    after the first call the second one allocates nothing, so it can be captured,
+    and the first one's graph stays valid."""
+    rng = np.random.default_rng(3)
+    beta = torch.tensor((10.0 ** rng.uniform(-1, 1, 16)).astype(np.float32)).cuda()
+    goals = torch.tensor(rng.uniform(0, 8, (16, 2)).astype(np.float32)).cuda()
+    obs = torch.tensor((3.0 + np.cumsum(rng.normal(0.0, 0.05, (65, 2)), 0)).astype(np.float32)).cuda()
+
+    def calls(G, B, n_obs):
+        held = goals[:G].contiguous(), beta[:B].contiguous()
+        model = pm.make_model(20, 1.0, 0.05, *held)
+        prior = torch.full((G * B,), float(-np.log(G * B))).cuda()
+        post = torch.empty_like(prior)
+        return post, held, lambda ctx: pm.pm_update_posterior_into(ctx, model, obs, n_obs, prior, post,
+                                                                   torch.cuda.current_stream())
+
+    few, many = calls(2, 2, 64), calls(16, 16, 1)
+    wants = []
+    for post, _, f in (few, many):
+        ctx = pm.pm_create(0)
+        f(ctx)
+        pm.pm_sync_status(ctx)
+        wants.append(post.clone())
+        pm.pm_destroy(ctx)
+    ctx = pm.pm_create(0)
+    try:
+        few[2](ctx)
+        torch.cuda.synchronize()
+        graphs = []
+        for post, _, f in (few, many):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                f(ctx)
+            graphs.append(g)
+        for g, (post, _, _), want in zip(graphs, (few, many), wants):
+            post.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(post, want)
+    finally:
+        pm.pm_destroy(ctx)
