@@ -370,12 +370,18 @@ float2 *fold_scratch(pm_ctx *ctx)
     return reinterpret_cast<float2 *>(reinterpret_cast<char *>(fast_rows(ctx)) + kFastRowBytes);
 }
 
+// A plain cudaMemset returns before it has run, on the legacy default stream,
+// and a non-blocking stream does not wait for that one: counters that kernels
+// find at zero and leave at zero are waited for once, where they are made.
+cudaError_t zeroed_for_every_stream() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 pm_status ensure_posterior_scratch(pm_ctx *ctx, size_t bytes)
 {
     if (!ctx->ticket) {
         // the counter block, the rows of the closed-form draw, the groups' folded components
         cudaError_t e = cudaMalloc((void **)&ctx->ticket, 256 + kFastRowBytes + pm::kMaxJ * sizeof(float2));
         if (e == cudaSuccess) e = cudaMemset(ctx->ticket, 0, 256);
+        if (e == cudaSuccess) e = zeroed_for_every_stream();
         if (e != cudaSuccess) {
             cudaGetLastError();
             ctx->ticket = nullptr;
@@ -1271,6 +1277,7 @@ pm_status pm_batch_create(pm_ctx *ctx, const pm_model *shared, int32_t max_human
     if (e == cudaSuccess) e = cudaMemset(b->d_prev, 0xFF, (size_t)max_humans * sizeof(float2));
     if (e == cudaSuccess) e = cudaMemset(reinterpret_cast<char *>(b->d_prev) + (size_t)max_humans * sizeof(float2), 0, 16);
     if (e == cudaSuccess) e = cudaMemset(b->d_meta, 0, 256);
+    if (e == cudaSuccess) e = zeroed_for_every_stream();
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->staged, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         cudaGetLastError();
