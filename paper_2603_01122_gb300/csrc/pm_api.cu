@@ -67,6 +67,7 @@ struct pm_batch {
     bool zero_reach = false;         // zero only the reachable cells (pm_batch_set_zeroing)
     float step_max = 0.0f;           // longest Euler step of the shared control set (upper bound)
     int t_max = 1;                   // longest horizon of the batch (sizes the zeroing grid)
+    int min_B = PM_MAX_COMPONENTS;   // fewest beta values of its humans
     pm::SmoothSrc *d_srcs = nullptr; // union source records, one per human
     uint8_t *d_flags = nullptr;      // block occupancy flags of every human's histogram
     size_t flags_cap = 0;
@@ -84,7 +85,7 @@ struct pm_batch {
     int n_items = 0;
     int max_chunks = 0;
     int max_J = 1;
-    int occ = 0; // resident CTAs per SM of the current shape (queried outside any capture)
+    int occ = 0, occ_rows = 0; // resident CTAs per SM of the current shape, without and with rows (queried outside any capture)
 };
 
 // A named NVTX range over one C ABI call, so that a profiler attributes the
@@ -282,6 +283,9 @@ void fill_rollout_tables(const pm_model *m, pm::RolloutArgs &a)
     a.fc.K = m->K;
 }
 
+// The enabled speeds of a control set (one speed: 1).
+int speeds_on(const pm::HeadingTab &t) { return t.S > 0 ? __builtin_popcount(t.speed_on) : 1; }
+
 // What builds the closed-form draw's rows at `rows`; rows == NULL (nothing to
 // build) where the control set does not take that draw.
 pm::FastPrep fast_prep(const pm_model *m, const pm::RolloutArgs &a, pm::FastRow *rows)
@@ -295,7 +299,7 @@ pm::FastPrep fast_prep(const pm_model *m, const pm::RolloutArgs &a, pm::FastRow 
     f.w1 = m->w1;
     f.w2 = m->w2;
     for (int q = 0; q < f.S; ++q) f.sl[q] = a.tab.S > 0 ? a.tab.sl[q] : a.tab.s;
-    f.rows = pm::fast_applies(m->K, a.enabled, __builtin_popcount(a.tab.speed_on)) ? rows : nullptr;
+    f.rows = pm::fast_applies(m->K, a.enabled, speeds_on(a.tab)) ? rows : nullptr;
     return f;
 }
 
@@ -465,8 +469,9 @@ pm_status predict_impl(pm_ctx *ctx, const pm_model *model, const float *log_beli
     const size_t words = hist ? (size_t)grid->W * (size_t)grid->H * (size_t)horizon : 0;
     // (the rollout leaves its chunk counter at zero; without `zero` the
     // caller has zeroed the outputs)
-    // a few steps do not repay the rows (2.5 us where the zeroing does not hide them)
-    const bool rows = model->B <= pm::kFastMaxB && horizon >= 8;
+    const bool rows = model->B <= pm::kFastMaxB &&
+                      pm::fast_pays(model->K, a.tab.S, speeds_on(a.tab), ((int64_t)n_particles + 31) / 32,
+                                    ctx->sm_count, horizon, !zero);
     const pm::FastPrep fp = fast_prep(model, a, rows ? fast_rows(ctx) : nullptr);
     a.fast = fp.rows;
     const bool z = zero && hist;
@@ -668,6 +673,19 @@ cudaError_t forget_starts(pm_batch *b, cudaStream_t stream)
     return cudaMemsetAsync(b->d_prev, 0xFF, (size_t)b->max_humans * sizeof(float2), stream);
 }
 
+// CTAs per SM of the batch's launch shape, without and with the closed-form draw.
+void set_occupancy(pm_batch *b)
+{
+    pm::RolloutArgs t;
+    std::memset(&t, 0, sizeof t);
+    fill_rollout_tables(&b->shared, t);
+    for (int rows = 0; rows < 2; ++rows)
+        (rows ? b->occ_rows : b->occ) =
+            pm::batch_rollout_occupancy(b->shared.K, t.enabled, t.tab.S, b->block_flags && b->warp_hist, rows != 0,
+                                        batch_shape_of(b), batch_dyn_smem(b));
+    cudaGetLastError();
+}
+
 pm_status batch_upload(pm_batch *b, cudaStream_t stream)
 {
     const int n = (int)b->humans.size();
@@ -787,9 +805,13 @@ pm_status batch_upload(pm_batch *b, cudaStream_t stream)
     char *p = b->h_stage;
     std::memcpy(p, hd.data(), bh);
     std::memcpy(p + bh, ph.data(), bp);
-    int t_max = 1;
-    for (const pm_human &u : b->humans) t_max = std::max(t_max, (int)u.horizon);
+    int t_max = 1, min_B = PM_MAX_COMPONENTS;
+    for (const pm_human &u : b->humans) {
+        t_max = std::max(t_max, (int)u.horizon);
+        min_B = std::min(min_B, (int)u.B);
+    }
     b->t_max = t_max;
+    b->min_B = min_B;
     int meta[3] = {(int)items.size(), n, t_max};
     std::memcpy(p + bh + bp, meta, sizeof meta);
     if (bi) std::memcpy(p + bh + bp + 16, items.data(), bi);
@@ -802,12 +824,7 @@ pm_status batch_upload(pm_batch *b, cudaStream_t stream)
     b->n_items = (int)items.size();
     b->max_chunks = std::max(b->max_chunks, max_chunks);
     b->max_J = std::max(b->max_J, max_J);
-    pm::RolloutArgs t;
-    std::memset(&t, 0, sizeof t);
-    fill_rollout_tables(&b->shared, t);
-    b->occ = pm::batch_rollout_occupancy(b->shared.K, t.enabled, t.tab.S, b->block_flags && b->warp_hist,
-                                         batch_shape_of(b), batch_dyn_smem(b));
-    cudaGetLastError();
+    set_occupancy(b);
     return PM_OK;
 }
 
@@ -817,6 +834,18 @@ pm_status batch_zero_impl(pm_batch *b, cudaStream_t stream)
                                           b->zero_reach ? b->d_prev : nullptr, zero_ticket(b), b->step_max, stream);
     if (e != cudaSuccess) return cuda_fail(e, "zero launch");
     return PM_OK;
+}
+
+// Whether a batch's launch takes the closed-form draw. A captured launch always
+// does: its graph may be given other humans before it is replayed.
+bool batch_rows_pay(const pm_batch *b, const pm::RolloutArgs &t, cudaStream_t stream)
+{
+    if (!b->d_fast || !b->warp_hist) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
+    else if (cap != cudaStreamCaptureStatusNone) return true;
+    return b->min_B <= pm::kFastMaxB && pm::fast_pays(b->shared.K, t.tab.S, speeds_on(t.tab), b->n_items,
+                                                      b->ctx->sm_count, b->t_max, true);
 }
 
 pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream, bool after_zero = false)
@@ -842,14 +871,14 @@ pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream, bool after_zero =
     a.status = status_word(ctx);
     a.marks = (b->block_flags && b->warp_hist && b->d_flags) ? 1 : 0;
     a.fc = t.fc;
-    const pm::FastPrep fp = fast_prep(&b->shared, t, b->warp_hist ? b->d_fast : nullptr);
+    const pm::FastPrep fp = fast_prep(&b->shared, t, batch_rows_pay(b, t, stream) ? b->d_fast : nullptr);
     if (fp.rows) {
         a.fast = fp.rows;
         e = pm::launch_batch_fast_rows(b->d_humans, b->d_meta + 1, b->max_humans, fp, after_zero, stream);
         if (e != cudaSuccess) return cuda_fail(e, "rows of the closed-form draw");
     }
     const size_t dyn = batch_dyn_smem(b);
-    int occ = b->occ;
+    int occ = fp.rows ? b->occ_rows : b->occ;
     if (occ < 1)
         return fail(PM_EINVAL, "launch shape (%d threads, %s) does not fit an SM", b->threads,
                     b->warp_hist ? "warp emplacement" : "shared window");
@@ -1491,12 +1520,7 @@ pm_status pm_batch_set_config(pm_batch *b, int32_t threads, int32_t shared_windo
     b->ctas_per_sm = ctas_per_sm;
     b->window_kib = window_kib;
     if (retile && !b->humans.empty()) return batch_upload(b, nullptr);
-    pm::RolloutArgs t;
-    std::memset(&t, 0, sizeof t);
-    fill_rollout_tables(&b->shared, t);
-    b->occ = pm::batch_rollout_occupancy(b->shared.K, t.enabled, t.tab.S, b->block_flags && b->warp_hist,
-                                         batch_shape_of(b), batch_dyn_smem(b));
-    cudaGetLastError();
+    set_occupancy(b);
     return PM_OK;
 }
 

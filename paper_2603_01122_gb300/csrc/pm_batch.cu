@@ -232,7 +232,7 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
         c.fbx = h->fbx;
         c.fplane = h->fbx * h->fby;
         if constexpr (MS)
-            rollout_lane<KT, false, true, true, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words, betas, a.K, h->speed_on);
+            rollout_lane<KT, false, true, FAST, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words, betas, a.K, h->speed_on);
         else rollout_lane<KT, FULL, false, FAST, false>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words);
     }
     release_counter(a.head, lane);
@@ -242,16 +242,18 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
 // per SM), and 72 (7 CTAs) for the one-speed instantiations with K <= 36,
 // which do not spill there (24 bytes with marks); the 64-human served frame
 // is 0.6 % faster with 7. K = 64 and several speeds spill at 72 and keep 80.
-template <int KT, bool FULL, bool MARKS = false>
+template <int KT, bool FULL, bool MARKS = false, bool MS = false>
 __global__ void __launch_bounds__(kBatchMaxThreads, 3) batch_warp_kernel(const __grid_constant__ BatchArgs a)
 {
-    batch_warp_body<KT, FULL, false, MARKS>(a);
+    batch_warp_body<KT, FULL, MS, MARKS>(a);
 }
 
 // With the closed-form draw. One speed, K <= 36: 80 registers (6 CTAs of 128
 // threads per SM; 96 registers and 5 CTAs: a frame of 64 humans 5.17 ms against
 // 4.91); K = 64 and several speeds: 96, for fewer spills (31 humans of 96
-// controls 2.06 ms against 2.26).
+// controls 2.06 ms against 2.26). Without rows several speeds keep
+// batch_warp_kernel (a human of 1000 particles and 144 controls, 20 steps:
+// 357 us against 421).
 template <int KT, bool FULL, bool MS, bool MARKS>
 __global__ void __maxnreg__((MS || KT == 64) ? 96 : 80) batch_fast_kernel(const __grid_constant__ BatchArgs a)
 {
@@ -518,22 +520,27 @@ cudaError_t batch_shape(const BatchArgs &a, const RolloutShape &sh, int blocks, 
     return launch_or_query(batch_rollout_kernel<KT, FULL>, a, blocks, sh.threads, dyn, s, occ);
 }
 
-cudaError_t batch_dispatch(const BatchArgs &a, const RolloutShape &sh, int blocks, size_t dyn, cudaStream_t s, int *occ)
+// Several speeds: warp-combined emplacement only.
+template <int KT>
+cudaError_t batch_multi(const BatchArgs &a, bool rows, const RolloutShape &sh, int blocks, size_t dyn, cudaStream_t s,
+                        int *occ)
 {
-    if (a.tab.S > 0) { // several speeds: warp-combined emplacement only
+    if (rows)
+        return a.marks ? launch_or_query(batch_fast_kernel<KT, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
+                       : launch_or_query(batch_fast_kernel<KT, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
+    return a.marks ? launch_or_query(batch_warp_kernel<KT, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
+                   : launch_or_query(batch_warp_kernel<KT, false, false, true>, a, blocks, sh.threads, dyn, s, occ);
+}
+
+cudaError_t batch_dispatch(const BatchArgs &a, bool rows, const RolloutShape &sh, int blocks, size_t dyn, cudaStream_t s,
+                           int *occ)
+{
+    if (a.tab.S > 0) {
         switch (a.K) {
-        case 16:
-            return a.marks ? launch_or_query(batch_fast_kernel<16, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_fast_kernel<16, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
-        case 32:
-            return a.marks ? launch_or_query(batch_fast_kernel<32, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_fast_kernel<32, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
-        case 36:
-            return a.marks ? launch_or_query(batch_fast_kernel<36, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_fast_kernel<36, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
-        default:
-            return a.marks ? launch_or_query(batch_fast_kernel<0, false, true, true>, a, blocks, sh.threads, dyn, s, occ)
-                           : launch_or_query(batch_fast_kernel<0, false, true, false>, a, blocks, sh.threads, dyn, s, occ);
+        case 16: return batch_multi<16>(a, rows, sh, blocks, dyn, s, occ);
+        case 32: return batch_multi<32>(a, rows, sh, blocks, dyn, s, occ);
+        case 36: return batch_multi<36>(a, rows, sh, blocks, dyn, s, occ);
+        default: return batch_multi<0>(a, rows, sh, blocks, dyn, s, occ);
         }
     }
     const int KT = rollout_kt_for(a.K);
@@ -555,7 +562,7 @@ size_t batch_warp_tables_bytes(int threads, bool multi_speed)
     return (size_t)(threads / 32) * (multi_speed ? kWarpTableBytesMS : kWarpTableBytes);
 }
 
-int batch_rollout_occupancy(int K, uint64_t enabled, int S, bool marks, const RolloutShape &shape, size_t dyn)
+int batch_rollout_occupancy(int K, uint64_t enabled, int S, bool marks, bool rows, const RolloutShape &shape, size_t dyn)
 {
     BatchArgs a;
     a.K = K;
@@ -563,7 +570,7 @@ int batch_rollout_occupancy(int K, uint64_t enabled, int S, bool marks, const Ro
     a.tab.S = S;
     a.marks = marks ? 1 : 0;
     int n = 0;
-    if (batch_dispatch(a, shape, 0, dyn, nullptr, &n) != cudaSuccess) {
+    if (batch_dispatch(a, rows, shape, 0, dyn, nullptr, &n) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -572,7 +579,7 @@ int batch_rollout_occupancy(int K, uint64_t enabled, int S, bool marks, const Ro
 
 cudaError_t launch_batch_rollout(const BatchArgs &a, const RolloutShape &shape, int blocks, size_t dyn, cudaStream_t s)
 {
-    return batch_dispatch(a, shape, blocks, dyn, s, nullptr);
+    return batch_dispatch(a, a.fast != nullptr, shape, blocks, dyn, s, nullptr);
 }
 
 cudaError_t launch_zero_outputs(uint32_t *counts, size_t words, uint32_t *oob, int T, unsigned *head, int sm_count,

@@ -67,6 +67,29 @@ __host__ __device__ __forceinline__ bool fast_applies(int K, uint64_t enabled, i
     return K >= 16 && K * (S > 1 ? S : 1) >= kFastMinK && (enabled & all) == all;
 }
 
+// Whether a call is long enough to repay its rows. Building them is one serial
+// chain of some 4 us beside the zeroing and 6 to 8 us in a launch of its own
+// (which also costs the rollout its early launch); what a step gives back grows
+// with the weights that it need not form, and with the tiles per scheduler once
+// each has one. In units of what a step of the fused one-speed draw gives back
+// (K = 36, or one enabled speed of several with K = 32 or 36), other draws give
+// three, and four from 64 controls of several speeds. Both sides at the line,
+// rows / no rows in us, one human of N particles waited for:
+//   K = 36, N = 1000: 24 steps 37 / 35, 32 steps 41 / 40, 48 steps 50 / 51
+//   K = 36, N = 100,000: 5 steps 33 / 32, 8 steps 36 / 38
+//   K = 20, N = 1000: 8 steps 28 / 26, 12 steps 29 / 30, 16 steps 32 / 33
+//   3 x 32, N = 1000: 5 steps 36 / 33, 8 steps 39 / 43
+// and a batch of 4 humans of 8000 particles, one call after another:
+//   K = 36: 16 steps 37 / 41, K = 20: 8 steps 29 / 31, 3 x 32: 8 steps 40 / 47
+__host__ __forceinline__ bool fast_pays(int K, int speeds, int speeds_on, int64_t tiles, int sm_count, int steps,
+                                        bool own_launch)
+{
+    const bool fused = speeds_on <= 1 && (K == 36 || (speeds > 1 && K == 32));
+    const float gain = fused ? 1.0f : (speeds_on > 1 && K * speeds_on >= 64) ? 4.0f : 3.0f;
+    const float per_scheduler = (float)tiles / (4.0f * (float)(sm_count > 0 ? sm_count : 1));
+    return (float)steps * gain * fminf(fmaxf(per_scheduler, 1.0f), 4.0f) >= (own_launch ? 48.0f : 32.0f);
+}
+
 #ifdef __CUDA_ARCH__
 #define PM_FAST_SYNC() __syncthreads()
 #else

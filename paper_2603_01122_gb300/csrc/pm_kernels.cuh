@@ -212,7 +212,7 @@ cudaError_t launch_philox_blocks(uint64_t seed, uint32_t human, uint32_t purpose
 cudaError_t launch_sfu_probe(int op, int blocks, int threads, int iters, float *sink,
                              cudaStream_t s);
 cudaError_t launch_adjoint(const AdjointArgs &a, cudaStream_t s);
-int batch_rollout_occupancy(int K, uint64_t enabled, int S, bool marks, const RolloutShape &shape, size_t dyn);
+int batch_rollout_occupancy(int K, uint64_t enabled, int S, bool marks, bool rows, const RolloutShape &shape, size_t dyn);
 size_t batch_warp_tables_bytes(int threads, bool multi_speed); // dynamic shared memory of the warp form
 cudaError_t launch_batch_rollout(const BatchArgs &a, const RolloutShape &shape, int blocks, size_t dyn, cudaStream_t s);
 // prev == NULL: every cell; else the reachable cells of humans with a

@@ -116,3 +116,61 @@ def test_far_goals_equal_weight_by_weight(K, speeds, away):
     want = _predict(K, speeds, 0, goals, np.append(beta, np.float32(1.0)), wide.ravel(), *args)
     for a, b in zip(got, want):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("K,speeds,lines", [(36, None, (31, 32, 47, 48)), (20, None, (10, 11, 15, 16)),
+                                            (32, (0.5, 1.0, 1.5), (7, 8, 11, 12)), (36, (0.5, 1.0), (7, 8, 11, 12)),
+                                            (12, (0.5, 1.0, 1.5, 2.0), (10, 11, 15, 16))])
+@pytest.mark.parametrize("marks", [0, 1])
+def test_short_batches_and_captures(K, speeds, lines, marks):
+    """Horizons on either side of the lines from which rows are built, in a batch
+    and alone; and a graph captured on a short batch, replayed on a longer one."""
+    rng = np.random.default_rng(K)
+    n, B, N, W, H = 3, 9, 700, 41, 47
+    goals = [torch.tensor(rng.uniform(-4.0, 4.0, (2 + i, 2)).astype(np.float32)).cuda() for i in range(n)]
+    beta = torch.tensor((10.0 ** np.linspace(-2.0, 1.5, B)).astype(np.float32)).cuda()
+    belief = [torch.tensor(np.log(rng.dirichlet(np.ones(len(g) * B))).astype(np.float32)).cuda() for g in goals]
+    z0 = torch.zeros((n, 2), device="cuda")
+    grid = pm.make_grid(-2.0, -2.0, 0.1, W, H)
+    ctx = pm.pm_create(0)
+    batch = None
+    try:
+        model = pm.make_model(K, 1.0, 0.04, goals[0], beta, speeds=speeds)
+        batch = pm.pm_batch_create(ctx, model, n)
+        if marks:
+            pm.pm_batch_set_block_flags(batch, 1)
+        graph, stream = None, torch.cuda.Stream()
+        for T in lines:
+            counts = torch.empty((n, T, H, W), dtype=torch.int32, device="cuda")
+            oob = torch.empty((n, T), dtype=torch.int32, device="cuda")
+            torch.cuda.synchronize()
+            pm.pm_batch_set(batch, [pm.make_human(goals[i], beta, belief[i], z0[i], N, T, grid, 7, i, counts[i], oob[i])
+                                    for i in range(n)], stream)
+            want = []
+            for i in range(n):
+                c, o = torch.empty_like(counts[0]), torch.empty_like(oob[0])
+                one = pm.make_model(K, 1.0, 0.04, goals[i], beta, speeds=speeds)
+                pm.pm_predict_occupancy(ctx, one, belief[i], 0.0, 0.0, N, T, grid, 7, i, c, o, stream)
+                want.append((c, o))
+            runs = [lambda: pm.pm_batch_predict(batch, stream)]
+            stream.synchronize()
+            if graph is None:
+                pm.pm_batch_predict(batch, stream)
+                stream.synchronize()
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=stream):
+                    pm.pm_batch_predict(batch, stream)
+            with torch.cuda.stream(stream):
+                runs.append(graph.replay)
+                for run in runs:
+                    counts.fill_(-1)
+                    oob.fill_(-1)
+                    run()
+                    stream.synchronize()
+                    for i, (c, o) in enumerate(want):
+                        assert torch.equal(counts[i], c) and torch.equal(oob[i], o), (T, i)
+        pm.pm_sync_status(ctx)
+    finally:
+        if batch is not None:
+            pm.pm_batch_destroy(batch)
+        pm.pm_destroy(ctx)
