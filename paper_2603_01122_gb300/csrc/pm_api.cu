@@ -294,11 +294,12 @@ pm::FastPrep fast_prep(const pm_model *m, const pm::RolloutArgs &a, pm::FastRow 
     std::memset(&f, 0, sizeof f);
     f.beta = m->beta;
     f.B = m->B;
-    f.S = a.tab.S > 0 ? a.tab.S : 1;
     f.K = m->K;
     f.w1 = m->w1;
     f.w2 = m->w2;
-    for (int q = 0; q < f.S; ++q) f.sl[q] = a.tab.S > 0 ? a.tab.sl[q] : a.tab.s;
+    if (a.tab.S <= 0) f.sl[f.S++] = a.tab.s;
+    for (int q = 0; q < a.tab.S; ++q)
+        if ((a.tab.speed_on >> q) & 1u) f.sl[f.S++] = a.tab.sl[q];
     f.rows = pm::fast_applies(m->K, a.enabled, speeds_on(a.tab)) ? rows : nullptr;
     return f;
 }
@@ -871,7 +872,11 @@ pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream, bool after_zero =
     a.status = status_word(ctx);
     a.marks = (b->block_flags && b->warp_hist && b->d_flags) ? 1 : 0;
     a.fc = t.fc;
-    const pm::FastPrep fp = fast_prep(&b->shared, t, batch_rows_pay(b, t, stream) ? b->d_fast : nullptr);
+    pm::FastPrep fp = fast_prep(&b->shared, t, batch_rows_pay(b, t, stream) ? b->d_fast : nullptr);
+    if (t.tab.S > 0) { // every speed: the humans have their own masks
+        fp.S = t.tab.S;
+        std::copy(t.tab.sl, t.tab.sl + t.tab.S, fp.sl);
+    }
     if (fp.rows) {
         a.fast = fp.rows;
         e = pm::launch_batch_fast_rows(b->d_humans, b->d_meta + 1, b->max_humans, fp, after_zero, stream);

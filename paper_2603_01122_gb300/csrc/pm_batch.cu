@@ -425,7 +425,8 @@ __device__ __forceinline__ void build_rows(const FastPrep &fp, int row0)
     fast_row_build(fp, min(row, n - 1), row < n, ws[grp], threadIdx.x - grp * kFastGroup, kFastGroup);
 }
 
-// blockIdx.y strides over the humans, the x dimension covers kFastMaxB * S rows.
+// blockIdx.y strides over the humans, the x dimension covers kFastMaxB * S rows
+// (S and the step lengths in fp: all speeds of the batch).
 __global__ void __launch_bounds__(kRowThreads) batch_fast_rows_kernel(const BatchHuman *humans, const int *n_dev,
                                                                       const __grid_constant__ FastPrep fp)
 {
@@ -437,8 +438,13 @@ __global__ void __launch_bounds__(kRowThreads) batch_fast_rows_kernel(const Batc
         p.B = h.B;
         p.beta = h.beta;
         p.rows = fp.rows + (size_t)hh * kFastMaxB * fp.S;
+        if (fp.S > 1) { // the human's own speeds
+            p.S = 0;
+            for (int q = 0; q < fp.S; ++q)
+                if ((h.speed_on >> q) & 1u) p.sl[p.S++] = fp.sl[q];
+        }
         const int row0 = blockIdx.x * kRowsPerCta;
-        if (h.B <= kFastMaxB && row0 < h.B * fp.S) build_rows(p, row0); // the same for the whole CTA
+        if (h.B <= kFastMaxB && row0 < h.B * p.S) build_rows(p, row0); // the same for the whole CTA
     }
     pdl_release();
 }

@@ -51,10 +51,10 @@ struct __align__(16) FastRow {
 
 struct FastPrep {
     const float *beta;
-    int B, S;                    // rows b * S + q, b < B <= kFastMaxB
+    int B, S;                    // rows b * S + q, b < B <= kFastMaxB, q the rank of a speed among the enabled ones
     int K;
     float w2, w1;                // Q weights
-    float sl[PM_MAX_SPEEDS];     // step lengths (one speed: sl[0])
+    float sl[PM_MAX_SPEEDS];     // step lengths of the enabled speeds (one speed: sl[0])
     FastRow *rows;
 };
 

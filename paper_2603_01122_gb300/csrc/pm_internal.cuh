@@ -235,7 +235,7 @@ struct RolloutArgs {
     int win_x0, win_y0;  // shared-memory window origin (grid cells)
     int win_side;        // window width | height << 16 (cells, each <= 255); 0 = no window
     FastConst fc;
-    const FastRow *fast; // rows of the closed-form draw (b * S + q), or NULL
+    const FastRow *fast; // rows of the closed-form draw (FastPrep), or NULL
     int n_trace;
     float *tr_states;
     uint8_t *tr_head;

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
         betas[j] = a.beta[b];
     }
     if (a.fast)
-        for (int i = tid; i < a.B * a.tab.S * (int)(sizeof(FastRow) / 16); i += blockDim.x)
+        for (int i = tid; i < a.B * __popc(a.tab.speed_on) * (int)(sizeof(FastRow) / 16); i += blockDim.x)
             fast_sm[i] = reinterpret_cast<const float4 *>(a.fast)[i];
     for (int u = tid; u < a.tab.S * a.K; u += blockDim.x)
         step[u] = make_float2(a.tab.msx[u / a.K][u % a.K], a.tab.msy[u / a.K][u % a.K]);
@@ -179,7 +179,7 @@ template <int KT, bool TRACE>
 cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
     int n = 0;
-    const size_t dyn = a.fast ? (size_t)a.B * a.tab.S * sizeof(FastRow) : 0;
+    const size_t dyn = a.fast ? (size_t)a.B * __builtin_popcount(a.tab.speed_on) * sizeof(FastRow) : 0;
     cudaError_t e = cudaFuncSetAttribute(rollout_multi_kernel<KT, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(kFastMaxB * PM_MAX_SPEEDS * sizeof(FastRow)));
     if (e != cudaSuccess) return e;

@@ -958,7 +958,7 @@ struct TileCtx {
     float *tr_states;
     uint8_t *tr_head;
     int32_t *tr_comp;
-    const FastRow *fast; // the human's rows of the closed-form draw (b * S + q), or NULL (rollout_lane)
+    const FastRow *fast; // the human's rows of the closed-form draw (FastPrep), or NULL (rollout_lane)
     int B;
     uint8_t *flags; // block occupancy [T][fby][fbx] (warp emplacement), or NULL
     int fbx;
@@ -1188,17 +1188,17 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
         if (trc && c.tr_comp) c.tr_comp[i] = lo;
         if constexpr (FAST) {
             if (c.fast) {
-                row = c.fast + (size_t)(lo % c.B) * (MS ? tab.S : 1);
+                const int nrow = MS ? __popc(speed_on) : 1; // of one beta: a row per enabled speed
+                row = c.fast + (size_t)(lo % c.B) * nrow;
                 float rmin = 0.0f; // the goal distance below which a row no longer holds
                 float smax = 0.0f; // the longest step
                 if constexpr (MS) {
-                    for (int q = 0; q < tab.S; ++q)
-                        if ((speed_on >> q) & 1u) {
-                            const float rm = row[q].rho_max;
-                            rmin = fmaxf(rmin, rm > 0.0f ? row[q].s / rm : INFINITY);
-                            ftol_r = fmaxf(ftol_r, fabsf(row[q].kappa) / row[q].s);
-                            smax = fmaxf(smax, row[q].s);
-                        }
+                    for (int q = 0; q < nrow; ++q) {
+                        const float rm = row[q].rho_max;
+                        rmin = fmaxf(rmin, rm > 0.0f ? row[q].s / rm : INFINITY);
+                        ftol_r = fmaxf(ftol_r, fabsf(row[q].kappa) / row[q].s);
+                        smax = fmaxf(smax, row[q].s);
+                    }
                 } else {
                     smax = row->s;
                     rmin = row->rho_max > 0.0f ? row->s / row->rho_max : INFINITY;
@@ -1333,12 +1333,14 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                     int base = 0;
                     if constexpr (MS) {
                         float wq[PM_MAX_SPEEDS], total = 0.0f;
+                        const FastRow *rows[PM_MAX_SPEEDS], *next = row;
 #pragma unroll
                         for (int q = 0; q < PM_MAX_SPEEDS; ++q) {
                             wq[q] = 0.0f;
+                            rows[q] = next;
                             if (q >= tab.S || !((speed_on >> q) & 1u)) continue; // the same for the whole warp
                             const float rq = tab.sl[q] * ri;
-                            const float4 m = *reinterpret_cast<const float4 *>(row[q].a0);
+                            const float4 m = *reinterpret_cast<const float4 *>((next++)->a0);
                             wq[q] = fmaf(fmaf(fmaf(m.w, rq, m.z), rq, m.y), rq, m.x);
                             total += wq[q];
                         }
@@ -1350,12 +1352,12 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                         for (int q = 1; q < PM_MAX_SPEEDS; ++q) {
                             const bool in = v >= run && wq[q] > 0.0f;
                             sp = in ? q : sp;
+                            o = in ? rows[q] : o;
                             start = in ? run : start;
                             wsel = in ? wq[q] : wsel;
                             run += wq[q];
                         }
                         const float iw = fast_rcp(wsel);
-                        o = row + sp;
                         base = sp * K;
                         rho = o->s * ri;
                         kap = o->kappa;

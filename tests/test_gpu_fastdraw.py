@@ -174,3 +174,35 @@ def test_short_batches_and_captures(K, speeds, lines, marks):
         if batch is not None:
             pm.pm_batch_destroy(batch)
         pm.pm_destroy(ctx)
+
+
+@pytest.mark.parametrize("K,speeds", [(20, (0.25, 1.0, 1.5, 2.0)), (36, (0.25, 0.5, 1.0, 1.5)), (32, (0.5, 1.0, 1.5))])
+def test_batch_with_own_speed_masks(K, speeds):
+    """Each human of a batch disables other speeds; its rows are those of its own
+    enabled ones, as in the single-human call with that mask."""
+    rng = np.random.default_rng(K)
+    S, B, N, T, W, H = len(speeds), 7, 900, 40, 51, 45
+    masks = [m for m in range(1 << S) if m != (1 << S) - 1]
+    n = len(masks)
+    goals = [torch.tensor(rng.uniform(-5.0, 5.0, (2, 2)).astype(np.float32)).cuda() for _ in range(n)]
+    beta = torch.tensor((10.0 ** np.linspace(-2.0, 1.5, B)).astype(np.float32)).cuda()
+    belief = torch.full((2 * B,), float(-np.log(2 * B))).cuda()
+    z0 = torch.zeros((n, 2), device="cuda")
+    grid = pm.make_grid(-2.0, -2.0, 0.09, W, H)
+    counts = torch.empty((n, T, H, W), dtype=torch.int32, device="cuda")
+    oob = torch.empty((n, T), dtype=torch.int32, device="cuda")
+    ctx = pm.pm_create(0)
+    try:
+        batch = pm.pm_batch_create(ctx, pm.make_model(K, 1.0, 0.03, goals[0], beta, speeds=speeds), n)
+        pm.pm_batch_set(batch, [pm.make_human(goals[i], beta, belief, z0[i], N, T, grid, 7, i, counts[i], oob[i],
+                                              speed_off=masks[i]) for i in range(n)])
+        pm.pm_batch_predict(batch)
+        for i in range(n):
+            c, o = torch.empty_like(counts[0]), torch.empty_like(oob[0])
+            one = pm.make_model(K, 1.0, 0.03, goals[i], beta, speeds=speeds, speed_off=masks[i])
+            pm.pm_predict_occupancy(ctx, one, belief, 0.0, 0.0, N, T, grid, 7, i, c, o)
+            pm.pm_sync_status(ctx)
+            assert torch.equal(counts[i], c) and torch.equal(oob[i], o), masks[i]
+        pm.pm_batch_destroy(batch)
+    finally:
+        pm.pm_destroy(ctx)
