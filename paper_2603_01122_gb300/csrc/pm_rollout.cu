@@ -26,7 +26,7 @@
 // is binned with FP32 operations (x - x0) * inv_res and the lanes of the warp
 // that land in the same cell are combined (match.any) into one global
 // reduction per cell and step.
-// rollout_multi_kernel<KT, TRACE> is the same kernel for a control set of several
+// rollout_multi_kernel<KT, TRACE, SHARED> is the same kernel for a control set of several
 // speeds (controls = speeds x headings, Sec. IV-B): the fused per-speed draw
 // for K = KT, the general one for any K (KT = 0).
 #include <cuda_runtime.h>
@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(kWarpCtaThreads, (FAST && KT == 64) ? 5 : kWar
 
 // The same persistent warps for a control set of several speeds: KT > 0 is
 // the heading count of the fused draw (K == KT), KT = 0 the general draw.
-template <int KT, bool TRACE>
+// SHARED: each CTA copies the closed-form draw's rows to shared memory.
+template <int KT, bool TRACE, bool SHARED>
 __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     rollout_multi_kernel(const __grid_constant__ RolloutArgs a, unsigned *head)
 {
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     __shared__ float betas[kMaxJ];
     __shared__ uint32_t cdf[kMaxJ];
     __shared__ float2 step[PM_MAX_SPEEDS * kMaxK];
-    extern __shared__ float4 fast_sm[]; // the rows of the closed-form draw: a lane reads another one at each step
+    extern __shared__ float4 fast_sm[]; // the rows of the closed-form draw (SHARED): a lane reads another one at each step
     __shared__ uint32_t words[kWarpCtaThreads / 32 * kWarpWords];
     const int tid = threadIdx.x, lane = tid & 31;
     const int J = a.G * a.B;
@@ -128,7 +129,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
         if (bad_component(cbj, comp[j].y, comp[j].z)) flag_status(a.status, kStatusModel);
         betas[j] = a.beta[b];
     }
-    if (a.fast)
+    if (SHARED)
         for (int i = tid; i < a.B * __popc(a.tab.speed_on) * (int)(sizeof(FastRow) / 16); i += blockDim.x)
             fast_sm[i] = reinterpret_cast<const float4 *>(a.fast)[i];
     for (int u = tid; u < a.tab.S * a.K; u += blockDim.x)
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     c.tr_states = a.tr_states;
     c.tr_head = a.tr_head;
     c.tr_comp = a.tr_comp;
-    c.fast = a.fast ? reinterpret_cast<const FastRow *>(fast_sm) : nullptr;
+    c.fast = SHARED ? reinterpret_cast<const FastRow *>(fast_sm) : a.fast;
     c.B = a.B;
     c.flags = nullptr;
     c.fbx = c.fplane = 0;
@@ -178,13 +179,31 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
 template <int KT, bool TRACE>
 cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
+    auto k = rollout_multi_kernel<KT, TRACE, false>;
     int n = 0;
-    const size_t dyn = a.fast ? (size_t)a.B * __builtin_popcount(a.tab.speed_on) * sizeof(FastRow) : 0;
-    cudaError_t e = cudaFuncSetAttribute(rollout_multi_kernel<KT, TRACE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(kFastMaxB * PM_MAX_SPEEDS * sizeof(FastRow)));
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kWarpCtaThreads, 0);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, rollout_multi_kernel<KT, TRACE>, kWarpCtaThreads, dyn);
-    if (e != cudaSuccess) return e;
+    // The rows go to shared memory while that leaves as many CTAs resident
+    // (100k particles, 60 steps, 3 speeds x 10 beta: 131 us against 139 from
+    // global memory); beyond (3 x 13, 4 x 10 and more) a CTA less costs more
+    // than it gives (3 x 16: 149 us against 135, and 1627 against 1387 where
+    // beta is too large for the closed form).
+    size_t dyn = 0;
+    if (a.fast) {
+        auto ks = rollout_multi_kernel<KT, TRACE, true>;
+        const size_t bytes = (size_t)a.B * __builtin_popcount(a.tab.speed_on) * sizeof(FastRow);
+        int ns = 0;
+        e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kFastMaxB * PM_MAX_SPEEDS * sizeof(FastRow)));
+        if (e != cudaSuccess) return e;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ns, ks, kWarpCtaThreads, bytes);
+        if (e != cudaSuccess) return e;
+        if (ns >= n) {
+            k = ks;
+            n = ns;
+            dyn = bytes;
+        }
+    }
     if (occ) {
         *occ = n;
         return cudaSuccess;
@@ -194,7 +213,7 @@ cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cud
     int64_t blocks = (int64_t)sm_count * (n > 0 ? n : 1);
     if (need < blocks) blocks = need;
     cudaGetLastError();
-    return launch_early(rollout_multi_kernel<KT, TRACE>, (unsigned)blocks, kWarpCtaThreads, dyn, s, a, head);
+    return launch_early(k, (unsigned)blocks, kWarpCtaThreads, dyn, s, a, head);
 }
 
 template <int KT, bool TRACE>
