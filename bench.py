@@ -36,9 +36,6 @@ sys.path.insert(0, ROOT)
 
 import workloads  # noqa: E402
 
-# Warp instructions per warp-step of the rollout with the closed-form draw (ncu, smsp__inst_executed)
-ISSUE_PER_WARP_STEP = {"one speed": 239, "several speeds": 343}
-ISSUE_PEAK = 4 * 152 * 2.07e9  # one warp instruction per clock and scheduler
 METRIC = "particle-steps/s"
 
 
@@ -54,8 +51,8 @@ def _measured_peak(key, default):
 
 HBM_PEAK_GBS = _measured_peak("hbm_gbs", 6794.5)
 # every source the rollout kernels are compiled from (the public header
-# reaches them only through pm_limits.h; the traffic of a
-# committed ncu summary is used only while these are unchanged)
+# reaches them only through pm_limits.h; the counts of a
+# committed ncu summary are used only while these are unchanged)
 ROLLOUT_SOURCES = ["paper_2603_01122_gb300/csrc/pm_rollout.cu", "paper_2603_01122_gb300/csrc/pm_rollout_dev.cuh",
                    "paper_2603_01122_gb300/csrc/pm_internal.cuh", "include/pm_limits.h",
                    "paper_2603_01122_gb300/csrc/pm_fastdraw.cuh"]
@@ -63,9 +60,12 @@ ROLLOUT_SOURCES = ["paper_2603_01122_gb300/csrc/pm_rollout.cu", "paper_2603_0112
 
 # main-line workloads: generator and the rollout kernel that dominates it
 MAIN_WORKLOADS = {
-    "paper_scale": (workloads.paper_scale, "rollout_warp_kernel<36,true>"),
-    "multi_speed": (workloads.multi_speed, "rollout_multi_kernel<32>"),
+    "paper_scale": (workloads.paper_scale, "rollout_warp_kernel<36,true,true,false>"),
+    "multi_speed": (workloads.multi_speed, "rollout_multi_kernel<32,false,true>"),
 }
+# of this library, per step of either: the belief update, the zeroing of the
+# outputs, the rows of the closed-form draw, the rollout
+LAUNCHES_PER_STEP = 4
 
 
 def parse():
@@ -314,9 +314,9 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-def load_profile_traffic(kernel_hash, workload="paper_scale"):
-    """DRAM bytes per launch of the rollout kernel from the committed ncu summary,
-    if it was taken on the current kernel source."""
+def load_profile(kernel_hash, workload="paper_scale"):
+    """The committed ncu summary of the workload's rollout kernel (DRAM bytes and
+    warp instructions of one launch), if it was taken on the current sources."""
     p = os.path.join(ROOT, "profiles", f"rollout_{workload}.json")
     if not os.path.exists(p):
         return None
@@ -324,9 +324,17 @@ def load_profile_traffic(kernel_hash, workload="paper_scale"):
         d = json.load(open(p))
     except Exception:
         return None
-    if d.get("kernel_sources_hash") != kernel_hash:
-        return None
-    return d.get("dram_bytes_per_launch")
+    return d if d.get("kernel_sources_hash") == kernel_hash else None
+
+
+def issue_rates(profile, seconds, sm_count, sm_mhz):
+    """Achieved and peak warp instructions per second of a launch that ``profile``
+    counted and that took ``seconds``: one per clock and scheduler is the peak, at
+    the SM clock sampled meanwhile. (None, None) where nothing was counted on these
+    sources or no clock was sampled."""
+    if not profile or not profile.get("warp_instructions") or not sm_mhz:
+        return None, None
+    return profile["warp_instructions"] / seconds, 4 * sm_count * sm_mhz * 1e6
 
 
 def gpu_paths(pm, ctx, torch, dev, hu, n_steps, human_id, start=None):
@@ -363,9 +371,10 @@ def time_events(torch, stream, fn, reps):
     return e0.elapsed_time(e1) / reps
 
 
-def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
+def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak, sm_mhz):
     """Batched, serving, differentiation and small-case numbers (secondary
-    workloads; each quoted with its own unit)."""
+    workloads; each quoted with its own unit). ``issue_roofline_frac`` is null
+    where the instructions of that workload's launches have not been counted."""
     out = {}
 
     def want(name):
@@ -486,7 +495,7 @@ def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
                           "speedup_vs_plain": plain_ms / batch_ms, "autotune_s": tune_s,
                           "tuned": tuned,
                           "rate_vs_plain_small": steps / (batch_ms * 1e-3) / out["plain_small"]["particle_steps_per_s"],
-                          "issue_roofline_frac": steps / (batch_ms * 1e-3) / 32 * ISSUE_PER_WARP_STEP["one speed"] / ISSUE_PEAK,
+                          "issue_roofline_frac": None,
                           "union": {"ms": union_ms, "sigma_cells": 1.5, "bytes": union_bytes,
                                     "GB_per_s": union_bytes / (union_ms * 1e-3) / 1e9,
                                     "hbm_frac": union_bytes / (union_ms * 1e-3) / 1e9 / HBM_PEAK_GBS,
@@ -604,7 +613,7 @@ def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
                 "particle_steps_per_frame": ps, "particle_steps_per_s": ps / float(np.median(lat)),
                 "plain_path_ms_per_frame": plain_ms, "speedup_vs_plain": plain_ms / float(np.median(lat) * 1e3),
                 "rate_vs_plain_small": ps / float(np.median(lat)) / out["plain_small"]["particle_steps_per_s"],
-                "issue_roofline_frac": ps / float(np.median(lat)) / 32 * ISSUE_PER_WARP_STEP["one speed"] / ISSUE_PEAK}
+                "issue_roofline_frac": None}
             # the same frames with the grid epilogue (blur + max-union on the room grid) in the graph
             srv_u = Server(ctx, hu0.K, hu0.speed, hu0.dt, hu0.grid, max_live=64, n_particles=hu0.n_particles,
                            horizon=hu0.horizon, window=hu0.window, union_sigma=1.5)
@@ -688,8 +697,11 @@ def run_extra(args, pm, ctx, torch, dev, stream, sfu_peak):
             ms = time_events(torch, stream, ms_step, 20)
             u_on = hu.K * sum(1 for q in range(len(hu.speeds)) if not (hu.speed_off >> q) & 1)
             rate = hu.n_particles * hu.horizon / (ms * 1e-3)
+            # (over the whole prediction; the rollout's instructions are those of its own main-line workload)
+            prof = None if stationary else load_profile(sources_hash(ROLLOUT_SOURCES), "multi_speed")
+            got, most = issue_rates(prof, ms * 1e-3, pm.pm_device_info(ctx)["sm_count"], sm_mhz)
             out[name] = {"ms_per_prediction": ms, "particle_steps_per_s": rate, "controls_enabled": u_on,
-                         "issue_roofline_frac": rate / 32 * ISSUE_PER_WARP_STEP["several speeds"] / ISSUE_PEAK}
+                         "issue_roofline_frac": got / most if got else None}
 
     if want("table1"):
         # -- Table 1's configuration (1 human, n = 8192, |G| = 10, |B| = 5, |U| = 96,
@@ -812,7 +824,6 @@ def run_native(args):
     hu = make_hu()
     human_id = rank_human_id(hu.human_id, rank)
     K, N, T = hu.K, hu.n_particles, hu.horizon
-    U = K * sum(1 for q in range(len(hu.speeds)) if not (hu.speed_off >> q) & 1)  # enabled controls
     x0, y0, res, W, H = hu.grid
     goals = torch.tensor(hu.goals, device=dev)
     beta = torch.tensor(hu.beta, device=dev)
@@ -907,29 +918,14 @@ def run_native(args):
     ms_per_step = total_ms / args.steps
     value = job_throughput(world, N * T, ms_per_step * 1e-3)
 
-    # roofline of the dominant kernel (the rollout): algorithmic SFU results
-    # per launch (one exp + one sqrt per control and particle-step) / its
-    # event-timed duration
+    # roofline of the dominant kernel (the rollout): with the closed-form draw
+    # instruction issue bounds it. The count of one launch is ncu's, the duration
+    # is event-timed here, the peak is at the clock sampled here.
     roll_avg_s = statistics.mean(roll_ms) * 1e-3
-    # (the closed-form draw, K >= 20 headings or several speeds, forms neither:
-    # its rollout is bound by instruction issue, counted by ncu)
-    closed = hu.K >= 16 and U >= 20 and len(hu.beta) <= 16 and not getattr(hu, "heading_off", 0)
-    if closed:
-        instr = ISSUE_PER_WARP_STEP["several speeds" if U > hu.K else "one speed"]
-        achieved = instr * ((N + 31) // 32) * T / roll_avg_s / 1e9
-        peak = ISSUE_PEAK / 1e9
-        unit, source = "G warp instructions/s", "one per clock and scheduler, 152 SMs x 4 at 2070 MHz"
-        algorithmic = f"{instr} warp instructions per warp-step (ncu, profiles/rollout_paper_scale.md)"
-    else:
-        sfu_ops = 2.0 * U * N * T
-        achieved = sfu_ops / roll_avg_s / 1e9
-        peak = 2.0 / (1.0 / sfu["ex2"] + 1.0 / sfu["sqrt"]) / 1e9
-        unit = "G SFU results/s"
-        source = ("measured by pm_probe_sfu (ex2/sqrt 1:1 harmonic mean); "
-                  f"ex2 {sfu['ex2'] / 1e9:.1f}, sqrt {sfu['sqrt'] / 1e9:.1f}, rsqrt {sfu['rsqrt'] / 1e9:.1f} G/s")
-        algorithmic = f"2U SFU results (U = {U} controls: U ex2 + U sqrt) per particle-step"
-    khash = sources_hash(ROLLOUT_SOURCES)
-    traffic = load_profile_traffic(khash, args.workload)
+    clocks = clk.summary()
+    profile = load_profile(sources_hash(ROLLOUT_SOURCES), args.workload)
+    achieved, peak = issue_rates(profile, roll_avg_s, info["sm_count"], clocks["sm_mhz"])
+    traffic = profile["dram_bytes_per_launch"] if profile else None
 
     # e2e through the host-buffer entry point (pinned buffers)
     goals_h = torch.tensor(hu.goals).pin_memory()
@@ -984,15 +980,17 @@ def run_native(args):
             "scaling": "weak", "vs_baseline": None, "dtype": "f32",
             "data": "synthetic (seeded; observed history drawn from the model on the GPU)",
             "config": workload_config(hu, args.workload),
-            # per step: the belief update, the zeroing of the outputs, the rows of the closed-form draw, the rollout
-            "gpu_launches": (4 if closed else 3) * args.steps,
+            "gpu_launches": LAUNCHES_PER_STEP * args.steps,
             "wall_s": wall,
             "breakdown_ms": {"posterior": statistics.mean(post_ms), "rollout": statistics.mean(roll_ms)},
-            "roofline": {"bound": "alu", "kernel": kernel_name, "achieved": achieved,
-                         "peak": peak, "unit": unit, "frac": achieved / peak, "traffic": traffic,
-                         "peak_source": source, "algorithmic": algorithmic},
+            "roofline": {"bound": "alu", "kernel": kernel_name, "achieved": achieved and achieved / 1e9,
+                         "peak": peak and peak / 1e9, "unit": "G warp instructions/s",
+                         "frac": achieved and achieved / peak, "traffic": traffic,
+                         "peak_source": f"one per clock and scheduler: 4 x {info['sm_count']} SMs at the sampled SM clock",
+                         "algorithmic": f"warp instructions of one launch (ncu, profiles/rollout_{args.workload}.json; "
+                                        "null unless taken on these sources)"},
             "device": info,
-            "clocks": {**clk.summary(), "window": f"{pre} pre-roll steps + the timed region"},
+            "clocks": {**clocks, "window": f"{pre} pre-roll steps + the timed region"},
             "e2e": {"value": e2e_value, "unit": METRIC, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "api": "pm_predict_host_async (one prediction after another; each step's copy-out "
                            "overlaps the next step)", "steps": a_steps,
@@ -1001,7 +999,8 @@ def run_native(args):
         }
         extra = None
         if not args.no_extra:
-            extra = run_extra(args, pm, ctx, torch, dev, stream, 2.0 / (1.0 / sfu["ex2"] + 1.0 / sfu["sqrt"]))
+            extra = run_extra(args, pm, ctx, torch, dev, stream, 2.0 / (1.0 / sfu["ex2"] + 1.0 / sfu["sqrt"]),
+                              clocks["sm_mhz"])
             line["extra"] = extra
         if not args.no_cpu_baseline:
             threads = host_threads()
