@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kRowThreads) zero_outputs_kernel(uint32_t *cou
 {
     // Nothing before the wait: the buffers may have been the inputs of whatever
     // ran before, and the beta grid its output. The rows are built beside the
-    // zeroing (4.5 us, hidden where 24 MB are zeroed).
+    // zeroing (some 4 us, hidden where 24 MB are zeroed).
     pdl_wait();
     if ((int)blockIdx.x >= zblocks) {
         build_rows(fp, ((int)blockIdx.x - zblocks) * kRowsPerCta);

@@ -19,9 +19,11 @@
 //
 // The result is used only where x lies clear of a whole number by more than
 // the error of this evaluation and of the weight-by-weight draw together
-// (`tol` below); the lanes that are closer (at least 2 K tol of them: one in
-// 4600 or more at K = 36) take the weight-by-weight draw, so the chosen
-// heading is always the one that the fixed-point weights give. A goal so far
+// (`tol` below); the lanes that are closer (2 K tol of them: one in 4600 at
+// K = 36 and small kappa, one in 4000 at kappa = 2, in 750 at 2.5 and in 45 at
+// 3, where the table starts too far off on the improbable side) take the weight-by-weight
+// draw, so the chosen heading is always the one that the fixed-point weights
+// give. A goal so far
 // away that those weights lose bits keeps the weight-by-weight draw
 // (rollout_lane).
 #pragma once
@@ -36,7 +38,12 @@ constexpr int kFastGuess = 64;     // intervals of the F^-1 table
 constexpr int kFastQ = 12;         // quadrature intervals on [0, pi]: harmonic n is aliased by 24 - n only
 constexpr int kFastMaxB = 16;      // beta values with a row; models with more use the weight-by-weight draw
 constexpr int kFastMinK = 20;      // fewer controls: the weights themselves are as cheap
-constexpr float kFastMaxKappa = 3.0f; // beyond it eight harmonics are not enough
+// Beyond it eight harmonics are not enough: at 3 (beta = 100, w2 = 1 and a step
+// of 3 cm reach it) they are off by 3e-5 of the CDF. One lane whose beta lies
+// beyond keeps its whole warp on the weight-by-weight draw, and the components
+// of a warp are drawn independently: where 7 % of the belief is on such beta,
+// 0.93^32 = 10 % of the warps still take the closed form.
+constexpr float kFastMaxKappa = 3.0f;
 constexpr int kFastGroup = 64;     // threads that build one row
 
 // One (beta, speed): what a draw needs of it.

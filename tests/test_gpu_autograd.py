@@ -92,3 +92,25 @@ def test_value_without_grad_mode_takes_no_gradient_pass(ctx, monkeypatch, call, 
     with mode():
         got = _call(ctx, p, call)
     assert torch.equal(got, want) and not got.requires_grad
+
+
+@pytest.mark.parametrize("K,speeds", [(12, None), (36, None), (16, (0.5, 1.0, 1.5))])
+def test_value_grad_rounds_to_the_scaled_gradient(ctx, K, speeds):
+    """The FP64 gradient, scaled and rounded to FP32, is what pm_loglik_backward
+    writes, bit for bit; a NULL gradient is refused."""
+    p = _inputs()
+    model = pm.make_model(K, 1.0, 0.1, p["goals"], p["beta"], w1=0.7, w2=1.3, speeds=speeds)
+    args = (ctx, model, 2, p["offsets"], 20, p["traj"], p["log_prior"])
+    L, L_b = torch.empty(1).cuda(), torch.empty(1).cuda()
+    grad = torch.empty(7, dtype=torch.float64).cuda()
+    pm.pm_loglik_value_grad(*args, L, grad)
+    for g in (1.0, -2.5, 1e-3, 3.14159274, 1e30):
+        dg, dv, dw = torch.empty((2, 2)).cuda(), torch.empty(1).cuda(), torch.empty(2).cuda()
+        pm.pm_loglik_backward(*args, g, L_b, dg, dv, dw)
+        pm.pm_sync_status(ctx)
+        want = torch.cat([dg.ravel(), dv, dw])
+        got = (grad * torch.tensor(g, dtype=torch.float32).double().cuda()).float()
+        assert torch.equal(L, L_b) and torch.equal(got, want), g
+    with pytest.raises(pm.PmError, match="grad is NULL") as e:
+        pm.pm_loglik_value_grad(*args, L, None)
+    assert e.value.status == pm.PM_EINVAL
