@@ -185,7 +185,7 @@ __device__ __forceinline__ void batch_warp_body(const BatchArgs &a)
                 const int g = j / h->B, b = j - g * h->B;
                 const float cbj = h->beta[b] * a.w2_log2e;
                 const float gx = h->goals[2 * g], gy = h->goals[2 * g + 1];
-                comp[j] = make_float4(cbj, gx, gy, lb_flag(a.tab, cbj));
+                comp[j] = make_float4(cbj, gx, gy, comp_flags(a.tab, cbj, h->z0[0] - gx, h->z0[1] - gy, h->T));
                 bad = bad || bad_component(cbj, gx, gy);
                 if constexpr (MS) betas[j] = h->beta[b];
             }

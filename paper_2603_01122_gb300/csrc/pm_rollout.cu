@@ -60,7 +60,8 @@ __global__ void __launch_bounds__(kWarpCtaThreads, (FAST && KT == 64) ? 5 : kWar
     for (int j = tid; j < J; j += blockDim.x) {
         const int g = j / a.B, b = j - g * a.B;
         const float cbj = a.beta[b] * a.w2_log2e;
-        comp[j] = make_float4(cbj, a.goals[2 * g], a.goals[2 * g + 1], lb_flag(a.tab, cbj));
+        comp[j] = make_float4(cbj, a.goals[2 * g], a.goals[2 * g + 1],
+                              comp_flags(a.tab, cbj, a.z0x - a.goals[2 * g], a.z0y - a.goals[2 * g + 1], a.T));
         if (bad_component(cbj, comp[j].y, comp[j].z)) flag_status(a.status, kStatusModel);
     }
     for (int k = tid; k < step_entries(KT); k += blockDim.x) step[k] = make_float2(a.tab.sx[k], a.tab.sy[k]);
@@ -125,7 +126,8 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     for (int j = tid; j < J; j += blockDim.x) {
         const int g = j / a.B, b = j - g * a.B;
         const float cbj = a.beta[b] * a.w2_log2e;
-        comp[j] = make_float4(cbj, a.goals[2 * g], a.goals[2 * g + 1], lb_flag(a.tab, cbj));
+        comp[j] = make_float4(cbj, a.goals[2 * g], a.goals[2 * g + 1],
+                              comp_flags(a.tab, cbj, a.z0x - a.goals[2 * g], a.z0y - a.goals[2 * g + 1], a.T));
         if (bad_component(cbj, comp[j].y, comp[j].z)) flag_status(a.status, kStatusModel);
         betas[j] = a.beta[b];
     }

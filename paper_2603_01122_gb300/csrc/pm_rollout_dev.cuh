@@ -364,6 +364,20 @@ __device__ __forceinline__ float lb_flag(const HeadingTab &tab, float cb)
     return (fabsf(cb) * tab.lb_gap <= 1.0f) ? 1.0f : 0.0f;
 }
 
+// The flags of a component in the rollouts' tables: 1 where lb_flag holds, plus 2
+// where the closed form may draw at any step of a particle that starts at (x, y).
+// The bound-normalised draw's reference distance lies 2^-20 r beyond the bound
+// (lb_step_d), so the largest of its 23-bit weights is 2^(-|cb| 2^-20 r) smaller.
+// Up to half a bit is within the closed form's tolerance; where a particle may get
+// farther the closed form would be the more exact one, but not the same one.
+__device__ __forceinline__ float comp_flags(const HeadingTab &tab, float cb, float dx, float dy, int T)
+{
+    float smax = tab.S > 0 ? 0.0f : tab.s;
+    for (int q = 0; q < tab.S; ++q) smax = fmaxf(smax, tab.sl[q]);
+    const float far = sqrt_approx(fmaf(dx, dx, dy * dy)) + (float)T * smax;
+    return lb_flag(tab, cb) + (fabsf(cb) * far <= 0x1p19f ? 2.0f : 0.0f);
+}
+
 // A component's table entry must be finite (goal and beta w2 log2(e)).
 __device__ __forceinline__ bool bad_component(float cb, float gx, float gy) { return !isfinite(cb + gx + gy); }
 
@@ -1180,7 +1194,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
         cb = cc.x;
         gx = cc.y;
         gy = cc.z;
-        lb = cc.w != 0.0f;
+        lb = cc.w == 1.0f || cc.w == 3.0f;
         if constexpr (MS) {
             bt = betas[lo];
             cw = bt * tab.w1l[0]; // beta w1 v dt log2(e)
@@ -1191,16 +1205,13 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                 const int nrow = MS ? __popc(speed_on) : 1; // of one beta: a row per enabled speed
                 row = c.fast + (size_t)(lo % c.B) * nrow;
                 float rmin = 0.0f; // the goal distance below which a row no longer holds
-                float smax = 0.0f; // the longest step
                 if constexpr (MS) {
                     for (int q = 0; q < nrow; ++q) {
                         const float rm = row[q].rho_max;
                         rmin = fmaxf(rmin, rm > 0.0f ? row[q].s / rm : INFINITY);
                         ftol_r = fmaxf(ftol_r, fabsf(row[q].kappa) / row[q].s);
-                        smax = fmaxf(smax, row[q].s);
                     }
                 } else {
-                    smax = row->s;
                     rmin = row->rho_max > 0.0f ? row->s / row->rho_max : INFINITY;
                     ftol_r = fabsf(row->kappa) / row->s;
                     fkap = row->kappa;
@@ -1212,14 +1223,7 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                 // beta w2 r: the 2^-23 of the approximate square root times
                 // the 1.8e-3 of its correction's factor, and twice that
                 ftol_r *= 4e-10f * (float)fc.K;
-                // Its reference distance lies 2^-20 r beyond the bound
-                // (lb_step_d), so the largest of its 23-bit weights is
-                // 2^(-|cb| 2^-20 r) smaller. Up to half a bit is within the
-                // tolerance; where a particle may get farther the closed
-                // form would be the more exact one, but not the same one.
-                const float dx = x - gx, dy = y - gy;
-                const float far = sqrt_approx(fmaf(dx, dx, dy * dy)) + (float)c.T * smax;
-                if (!(fabsf(cb) * far <= 0x1p19f)) fr2 = INFINITY;
+                if (cc.w < 2.0f) fr2 = INFINITY; // comp_flags
             }
         }
     }
