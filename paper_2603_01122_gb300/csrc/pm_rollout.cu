@@ -26,7 +26,7 @@
 // is binned with FP32 operations (x - x0) * inv_res and the lanes of the warp
 // that land in the same cell are combined (match.any) into one global
 // reduction per cell and step.
-// rollout_multi_kernel<KT, TRACE, SHARED> is the same kernel for a control set of several
+// rollout_multi_kernel<KT, TRACE, SHARED, MASKED> is the same kernel for a control set of several
 // speeds (controls = speeds x headings, Sec. IV-B): the fused per-speed draw
 // for K = KT, the general one for any K (KT = 0).
 #include <cuda_runtime.h>
@@ -109,8 +109,9 @@ __global__ void __launch_bounds__(kWarpCtaThreads, (FAST && KT == 64) ? 5 : kWar
 
 // The same persistent warps for a control set of several speeds: KT > 0 is
 // the heading count of the fused draw (K == KT), KT = 0 the general draw.
-// SHARED: each CTA copies the closed-form draw's rows to shared memory.
-template <int KT, bool TRACE, bool SHARED>
+// SHARED: each CTA copies the closed-form draw's rows to shared memory. MASKED:
+// some speeds may be disabled.
+template <int KT, bool TRACE, bool SHARED, bool MASKED>
 __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
     rollout_multi_kernel(const __grid_constant__ RolloutArgs a, unsigned *head)
 {
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
         const int64_t i0 = (int64_t)item * 32;
         if (i0 >= a.N) break;
         c.i = i0 + lane;
-        rollout_lane<KT, false, true, true, TRACE>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words + (tid >> 5) * kWarpWords + lane, betas, a.K, a.tab.speed_on);
+        rollout_lane<KT, false, true, true, TRACE, MASKED>(a.tab, a.enabled, a.s2, a.fc, c, comp, cdf, step, words + (tid >> 5) * kWarpWords + lane, betas, a.K, a.tab.speed_on);
     }
     release_counter(head, lane);
 }
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(kWarpCtaThreads, kWarpCtaMinBlocks)
 template <int KT, bool TRACE>
 cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cudaStream_t s, int *occ)
 {
-    auto k = rollout_multi_kernel<KT, TRACE, false>;
+    auto k = rollout_multi_kernel<KT, TRACE, false, true>;
     int n = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kWarpCtaThreads, 0);
     if (e != cudaSuccess) return e;
@@ -192,7 +193,10 @@ cudaError_t launch_multi(const RolloutArgs &a, unsigned *head, int sm_count, cud
     // beta is too large for the closed form).
     size_t dyn = 0;
     if (a.fast) {
-        auto ks = rollout_multi_kernel<KT, TRACE, true>;
+        auto ks = rollout_multi_kernel<KT, TRACE, true, true>;
+        if constexpr (!TRACE) {
+            if (__builtin_popcount(a.tab.speed_on) == a.tab.S) ks = rollout_multi_kernel<KT, false, true, false>;
+        }
         const size_t bytes = (size_t)a.B * __builtin_popcount(a.tab.speed_on) * sizeof(FastRow);
         int ns = 0;
         e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -1162,7 +1162,9 @@ constexpr int kWarpWords = 8 * 32;
 // lane's row usable and its goal farther than the row's range), and weight by
 // weight for the lanes it leaves open and at every other step. A warp-wide
 // choice: with both forms in one step the warp would pay for both.
-template <int KT, bool FULL, bool MS, bool FAST, bool TRACE>
+// MASKED: some of the speeds may be disabled (without: 278 us instead of 281 for
+// 100k particles of 96 controls).
+template <int KT, bool FULL, bool MS, bool FAST, bool TRACE, bool MASKED = true>
 __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t enabled, float s2, const FastConst &fc,
                                              const TileCtx &c, const float4 *comp, const uint32_t *cdf,
                                              const float2 *step, uint32_t *words, const float *betas = nullptr, int K = 0,
@@ -1337,14 +1339,13 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                     int base = 0;
                     if constexpr (MS) {
                         float wq[PM_MAX_SPEEDS], total = 0.0f;
-                        const FastRow *rows[PM_MAX_SPEEDS], *next = row;
+                        int nr = 0; // enabled speeds before q: q's row
 #pragma unroll
                         for (int q = 0; q < PM_MAX_SPEEDS; ++q) {
                             wq[q] = 0.0f;
-                            rows[q] = next;
                             if (q >= tab.S || !((speed_on >> q) & 1u)) continue; // the same for the whole warp
                             const float rq = tab.sl[q] * ri;
-                            const float4 m = *reinterpret_cast<const float4 *>((next++)->a0);
+                            const float4 m = *reinterpret_cast<const float4 *>(row[MASKED ? nr++ : q].a0);
                             wq[q] = fmaf(fmaf(fmaf(m.w, rq, m.z), rq, m.y), rq, m.x);
                             total += wq[q];
                         }
@@ -1356,12 +1357,12 @@ __device__ __forceinline__ void rollout_lane(const HeadingTab &tab, uint64_t ena
                         for (int q = 1; q < PM_MAX_SPEEDS; ++q) {
                             const bool in = v >= run && wq[q] > 0.0f;
                             sp = in ? q : sp;
-                            o = in ? rows[q] : o;
                             start = in ? run : start;
                             wsel = in ? wq[q] : wsel;
                             run += wq[q];
                         }
                         const float iw = fast_rcp(wsel);
+                        o = row + (MASKED ? __popc(speed_on & ((1u << sp) - 1u)) : sp);
                         base = sp * K;
                         rho = o->s * ri;
                         kap = o->kappa;
