@@ -6,9 +6,9 @@
 // Where every heading is enabled and there are 20 controls or more, most steps
 // draw the heading in closed form (pm_fastdraw.cuh): 239 warp instructions per
 // warp-step at K = 36 instead of 411, 343 at 96 controls instead of 1262; the
-// launch is then bound by instruction issue (63 % of the slots with 100k
-// particles, 75 % with many humans), the special-function unit no longer.
-// 100k particles, K = 36, 150 steps: 295 -> 169 us; 96 controls: 871 -> 253.
+// launch is then bound by instruction issue (64 % of the slots with 100k
+// particles, 74 % with many humans), the special-function unit no longer.
+// 100k particles, K = 36, 150 steps: 295 -> 167 us; 96 controls: 871 -> 258.
 //
 // Weight by weight, per particle and step, for every heading k:
 //   distance from the next state to the goal, d_k = sqrt(D + 2 s e_k.(z - g))
