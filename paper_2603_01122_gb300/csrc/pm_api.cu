@@ -680,10 +680,12 @@ void set_occupancy(pm_batch *b)
     pm::RolloutArgs t;
     std::memset(&t, 0, sizeof t);
     fill_rollout_tables(&b->shared, t);
-    for (int rows = 0; rows < 2; ++rows)
-        (rows ? b->occ_rows : b->occ) =
-            pm::batch_rollout_occupancy(b->shared.K, t.enabled, t.tab.S, b->block_flags && b->warp_hist, rows != 0,
-                                        batch_shape_of(b), batch_dyn_smem(b));
+    auto query = [&](bool rows) {
+        return pm::batch_rollout_occupancy(b->shared.K, t.enabled, t.tab.S, b->block_flags && b->warp_hist, rows,
+                                           batch_shape_of(b), batch_dyn_smem(b));
+    };
+    b->occ = query(false);
+    b->occ_rows = t.tab.S > 0 ? query(true) : b->occ; // one speed: the same kernel
     cudaGetLastError();
 }
 
