@@ -19,13 +19,12 @@
 //
 // The result is used only where x lies clear of a whole number by more than
 // the error of this evaluation and of the weight-by-weight draw together
-// (`tol` below); the lanes that are closer (2 K tol of them: one in 4600 at
-// K = 36 and small kappa, one in 4000 at kappa = 2, in 750 at 2.5 and in 45 at
-// 3, where the table starts too far off on the improbable side) take the weight-by-weight
-// draw, so the chosen heading is always the one that the fixed-point weights
-// give. A goal so far
-// away that those weights lose bits keeps the weight-by-weight draw
-// (rollout_lane).
+// (`tol` below); the lanes that are closer take the weight-by-weight draw, so
+// the chosen heading is always the one that the fixed-point weights give. They
+// are 2 K tol of the draws: one in 4600 at K = 36 and small kappa, one in 4000
+// at kappa = 2, in 750 at 2.5 and in 45 at 3, where the table starts too far
+// off on the improbable side. A goal so far away that those weights lose bits
+// keeps the weight-by-weight draw (comp_flags).
 #pragma once
 
 #include "pm_internal.cuh"
