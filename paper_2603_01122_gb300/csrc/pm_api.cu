@@ -847,8 +847,8 @@ bool batch_rows_pay(const pm_batch *b, const pm::RolloutArgs &t, cudaStream_t st
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
     else if (cap != cudaStreamCaptureStatusNone) return true;
-    return b->min_B <= pm::kFastMaxB && pm::fast_pays(b->shared.K, t.tab.S, speeds_on(t.tab), b->n_items,
-                                                      b->ctx->sm_count, b->t_max, true);
+    return b->min_B <= pm::kFastMaxB && pm::fast_pays_batch(b->shared.K, t.tab.S, speeds_on(t.tab), b->n_items,
+                                                            b->ctx->sm_count, b->t_max);
 }
 
 pm_status batch_rollout_impl(pm_batch *b, cudaStream_t stream, bool after_zero = false)

@@ -73,27 +73,52 @@ __host__ __device__ __forceinline__ bool fast_applies(int K, uint64_t enabled, i
     return K >= 16 && K * (S > 1 ? S : 1) >= kFastMinK && (enabled & all) == all;
 }
 
-// Whether a call is long enough to repay its rows. Building them is one serial
-// chain of some 4 us beside the zeroing and 6 to 8 us in a launch of its own
-// (which also costs the rollout its early launch); what a step gives back grows
-// with the weights that it need not form, and with the tiles per scheduler once
-// each has one. In units of what a step of the fused one-speed draw gives back
-// (K = 36, or one enabled speed of several with K = 32 or 36), other draws give
-// three, and four from 64 controls of several speeds. Both sides at the line,
-// rows / no rows in us, one human of N particles waited for:
+// Whether one human's call is long enough to repay its rows. Building them is
+// one serial chain of some 4 us beside the zeroing and 6 us in a launch of its
+// own (own_launch); what a step gives back grows with the weights that it need
+// not form, and with the tiles per scheduler once each has one. In units of what
+// a step of the fused one-speed draw gives back (K = 36, or one enabled speed of
+// several with K = 32 or 36), other draws give three, and four from 64 controls
+// of several speeds. Both sides at the line, rows / no rows in us, one human of
+// N particles waited for:
 //   K = 36, N = 1000: 24 steps 37 / 35, 32 steps 41 / 40, 48 steps 50 / 51
 //   K = 36, N = 100,000: 5 steps 33 / 32, 8 steps 36 / 38
 //   K = 20, N = 1000: 8 steps 28 / 26, 12 steps 29 / 30, 16 steps 32 / 33
 //   3 x 32, N = 1000: 5 steps 36 / 33, 8 steps 39 / 43
-// and a batch of 4 humans of 8000 particles, one call after another:
-//   K = 36: 16 steps 37 / 41, K = 20: 8 steps 29 / 31, 3 x 32: 8 steps 40 / 47
+__host__ __forceinline__ bool fast_fused(int K, int speeds, int speeds_on)
+{
+    return speeds_on <= 1 && (K == 36 || (speeds > 1 && K == 32));
+}
+
 __host__ __forceinline__ bool fast_pays(int K, int speeds, int speeds_on, int64_t tiles, int sm_count, int steps,
                                         bool own_launch)
 {
-    const bool fused = speeds_on <= 1 && (K == 36 || (speeds > 1 && K == 32));
-    const float gain = fused ? 1.0f : (speeds_on > 1 && K * speeds_on >= 64) ? 4.0f : 3.0f;
+    const float gain = fast_fused(K, speeds, speeds_on) ? 1.0f : (speeds_on > 1 && K * speeds_on >= 64) ? 4.0f : 3.0f;
     const float per_scheduler = (float)tiles / (4.0f * (float)(sm_count > 0 ? sm_count : 1));
     return (float)steps * gain * fminf(fmaxf(per_scheduler, 1.0f), 4.0f) >= (own_launch ? 48.0f : 32.0f);
+}
+
+// The same for a batch, whose rows take a launch of their own and cost the
+// rollout its early launch (8 us). From 100 tiles on several warps share a
+// scheduler (a CTA takes four tiles at a time), and a step gives back twice as
+// much; beyond six tiles per scheduler it grows with them. The line lies half
+// above the break-even: where no warp can use the rows (|kappa| > 3, which the
+// host does not see) the 8 us are lost. Rows / no rows in us, one call after
+// another, humans x particles:
+//   K = 36: 1 x 1000, 32 steps 39 / 40, 64 steps 59 / 71; 4 x 1000, 16 steps
+//     33 / 35, 24 steps 40 / 48; 16 x 8000, 16 steps 48 / 49, 24 steps 58 / 66
+//   K = 20: 4 x 1000, 8 steps 26 / 26, 12 steps 30 / 35; 64 x 8000, 5 steps 63 / 80
+//   K = 64: 4 x 1000, 8 steps 27 / 30, 12 steps 31 / 40
+//   2 x 16: 4 x 1000, 12 steps 33 / 33, 16 steps 36 / 41; 16 x 8000, 12 steps 63 / 63
+//   3 x 32: 1 x 1000, 8 steps 33 / 35, 16 steps 38 / 59; 4 x 8000, 8 steps 40 / 47
+__host__ __forceinline__ bool fast_pays_batch(int K, int speeds, int speeds_on, int64_t tiles, int sm_count, int steps)
+{
+    const float gain = fast_fused(K, speeds, speeds_on) ? 1.0f
+                       : speeds_on > 1 ? (float)(K * speeds_on) * (1.0f / 32.0f) + 0.5f
+                       : (K <= 24 || K == 64) ? 2.0f
+                                              : 4.0f;
+    const float per_scheduler = (float)tiles / (4.0f * (float)(sm_count > 0 ? sm_count : 1));
+    return (float)steps * gain * fmaxf(tiles >= 100 ? 2.0f : 1.0f, per_scheduler * (1.0f / 3.0f)) >= 48.0f;
 }
 
 #ifdef __CUDA_ARCH__

@@ -118,9 +118,10 @@ def test_far_goals_equal_weight_by_weight(K, speeds, away):
         assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("K,speeds,lines", [(36, None, (31, 32, 47, 48)), (20, None, (10, 11, 15, 16)),
-                                            (32, (0.5, 1.0, 1.5), (7, 8, 11, 12)), (36, (0.5, 1.0), (7, 8, 11, 12)),
-                                            (12, (0.5, 1.0, 1.5, 2.0), (10, 11, 15, 16))])
+@pytest.mark.parametrize("K,speeds,lines", [(36, None, (31, 32, 47, 48)), (20, None, (10, 11, 15, 16, 23, 24)),
+                                            (32, (0.5, 1.0, 1.5), (7, 8, 11, 12, 13, 14)),
+                                            (36, (0.5, 1.0), (7, 8, 11, 12, 17, 18)),
+                                            (12, (0.5, 1.0, 1.5, 2.0), (10, 11, 15, 16, 23, 24))])
 @pytest.mark.parametrize("marks", [0, 1])
 def test_short_batches_and_captures(K, speeds, lines, marks):
     """Horizons on either side of the lines from which rows are built, in a batch
