@@ -3,17 +3,17 @@
 ``MarginalLogLik.apply(goals, speed, w, beta, K, dt, offsets, traj, log_prior, ctx, speeds, snap_heading)``
 returns the marginal log-likelihood L of the observed trajectories (a CUDA
 scalar). Where a gradient is wanted (an input requires one and the grad mode is
-on), the forward call takes L and the gradient
-with respect to the goal coordinates, the speed and the Q weights from one
-pass of the adjoint kernel (it forms both from the same weights; a second
-pass in backward cost as much again), and backward scales it on the device,
-in FP64 before the rounding to FP32. An incoming gradient that is not finite
-is refused (PM_EINVAL), as pm_loglik_backward refuses it.
-``speed`` and ``w`` are read to the host once per call (the C ABI takes them
-as scalars). ``speeds`` (a tuple of multipliers, or None for one speed)
-selects the control set of several speeds; ``snap_heading`` reads each
-observed heading as the nearest enabled heading. 256 trajectories, G = 4,
-B = 10, value and gradient waited for: 465 -> 395 us, a value alone 154.
+on), the forward call takes L and the gradient with respect to the goal
+coordinates, the speed and the Q weights from one pass of the adjoint kernel (it
+forms both from the same weights; a second pass in backward cost as much again),
+and backward scales it on the device, in FP64 before the rounding to FP32. An
+incoming gradient that is not finite is refused (PM_EINVAL), as
+pm_loglik_backward refuses it. ``speed`` and ``w`` are read to the host once per
+call (the C ABI takes them as scalars), the incoming gradient once in backward.
+``speeds`` (a tuple of multipliers, or None for one speed) selects the control
+set of several speeds; ``snap_heading`` reads each observed heading as the
+nearest enabled heading. 256 trajectories, G = 4, B = 10, value and gradient
+waited for: 440 -> 357 us, a value alone 152.
 """
 from __future__ import annotations
 
@@ -68,9 +68,12 @@ class MarginalLogLik(torch.autograd.Function):
     @staticmethod
     def backward(fctx, grad_out):
         grad, goals, speed, w = fctx.saved_tensors[:4]
+        g = grad_out.item()  # one read; it also makes the scaling by 1 of a plain backward() unnecessary
+        if not math.isfinite(g):
+            raise PmError(PM_EINVAL, "grad_out must be finite")
         out = [None] * len(fctx.needs_input_grad)
         if grad is not None:
-            d = (grad * grad_out.detach()).to(torch.float32)  # the product in FP64
+            d = (grad if g == 1.0 else grad * g).to(torch.float32)  # the product in FP64
             n = goals.numel()
             need = fctx.needs_input_grad
             if need[0]:
@@ -79,9 +82,6 @@ class MarginalLogLik(torch.autograd.Function):
                 out[1] = d[n:n + 1].to(speed.device).reshape(speed.shape)
             if need[2]:
                 out[2] = d[n + 1:].to(w.device).reshape(w.shape)
-        # read back after the work above is queued: what waits for it is the check alone
-        if not math.isfinite(grad_out.item()):
-            raise PmError(PM_EINVAL, "grad_out must be finite")
         return tuple(out)
 
 
